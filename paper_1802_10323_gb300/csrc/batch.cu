@@ -33,20 +33,15 @@
 
 namespace ps {
 
-template <class T>
-int pick_lines(int n, int axis, int nx, int nlines);
-
 enum BStage { BS_XF64 = 0, BS_XF, BS_YF, BS_Z, BS_ZS, BS_YB, BS_XBST, BS_XBACC, BS_RES, BS_CHK, BS_FIN };
 
 struct BGrid {
   int nx, ny, nz, bcx, bcy, bcz, singular, periodic_z;
-  int mx, my, nstx, nsty;
-  int radx[kMaxStages], rady[kMaxStages];
-  int Lx, Ly;              // lines per transform task
+  int mx, my;
+  int lgx, lgy;            // log2 of the lines per transform task
   int res_chunk;           // points per residual task
   int ntask[4];            // x tasks, y tasks, z tasks, residual tasks
-  const cplx<float>* twx;
-  const cplx<float>* twy;
+  LineTab<float> tabx, taby;
   const float *lamx, *lamy, *za, *zb, *zc, *dzf;
   const float2 *zlo, *zhi;
   df idx2, idy2;
@@ -89,13 +84,9 @@ __device__ XformArgs<float> bx_args(const BGrid& G, int axis, const void* in, vo
   a.ny = G.ny;
   a.nz = G.nz;
   if (axis == 0) {
-    a.n = 2 * G.mx; a.m = G.mx; a.L = G.Lx; a.nlines = G.ny * G.nz; a.bc = G.bcx;
-    a.nstages = G.nstx; a.tw = G.twx;
-    for (int i = 0; i < kMaxStages; ++i) a.radix[i] = G.radx[i];
+    a.n = 2 * G.mx; a.m = G.mx; a.lgL = G.lgx; a.nlines = G.ny * G.nz; a.bc = G.bcx; a.tab = G.tabx;
   } else {
-    a.n = 2 * G.my; a.m = G.my; a.L = G.Ly; a.nlines = G.nx * G.nz; a.bc = G.bcy;
-    a.nstages = G.nsty; a.tw = G.twy;
-    for (int i = 0; i < kMaxStages; ++i) a.radix[i] = G.rady[i];
+    a.n = 2 * G.my; a.m = G.my; a.lgL = G.lgy; a.nlines = G.nx * G.nz; a.bc = G.bcy; a.tab = G.taby;
   }
   a.plane_scale = nullptr;
   a.accumulate = acc;
@@ -305,13 +296,13 @@ __global__ void __launch_bounds__(256, 4) batch_kernel(BatchArgs A) {
       float* partial = reinterpret_cast<float*>(ws + G.ws_off);
       switch (type) {
         case BS_XF64:
-          xform_group<float, double, float, true>(bx_args(G, 0, A.f[g], w, 0, nullptr), idx, smem);
+          xform_group<float, double, float, true, 9>(bx_args(G, 0, A.f[g], w, 0, nullptr), idx, smem);
           break;
         case BS_XF:
-          xform_group<float, float, float, true>(bx_args(G, 0, w, w, 0, nullptr), idx, smem);
+          xform_group<float, float, float, true, 9>(bx_args(G, 0, w, w, 0, nullptr), idx, smem);
           break;
         case BS_YF:
-          xform_group<float, float, float, true>(bx_args(G, 1, w, w, 0, nullptr), idx, smem);
+          xform_group<float, float, float, true, 9>(bx_args(G, 1, w, w, 0, nullptr), idx, smem);
           break;
         case BS_Z:
           zsolve_column<float>(bz_args(G, ws), idx * blockDim.x + threadIdx.x);
@@ -320,14 +311,14 @@ __global__ void __launch_bounds__(256, 4) batch_kernel(BatchArgs A) {
           zsingular_block<float>(bz_args(G, ws), smem);
           break;
         case BS_YB:
-          xform_group<float, float, float, false>(bx_args(G, 1, w, w, 0, nullptr), idx, smem);
+          xform_group<float, float, float, false, 9>(bx_args(G, 1, w, w, 0, nullptr), idx, smem);
           break;
         case BS_XBST:
           if (idx == 0 && threadIdx.x == 0) reset_red(c);
-          xform_group<float, float, double, false>(bx_args(G, 0, w, A.p[g], 0, nullptr), idx, smem);
+          xform_group<float, float, double, false, 9>(bx_args(G, 0, w, A.p[g], 0, nullptr), idx, smem);
           break;
         case BS_XBACC:
-          xform_group<float, float, double, false>(bx_args(G, 0, w, A.p[g], 1, nullptr), idx, smem);
+          xform_group<float, float, double, false, 9>(bx_args(G, 0, w, A.p[g], 1, nullptr), idx, smem);
           break;
         case BS_RES:
         case BS_CHK:
@@ -409,6 +400,11 @@ bool is_candidate_scale(int sc) {
   return false;
 }
 
+// shared memory of a tile of 2^lg lines (xform_group)
+size_t batch_tile_smem(int m, int lg) {
+  return 2 * (size_t)(m + 1) * (lg ? ((size_t)1 << lg) + 1 : 1) * sizeof(cplx<float>);
+}
+
 // Build the device tables for the current tile scale.
 ps_status build_tables(ps_batch* b) {
   if (b->dev) {
@@ -447,28 +443,27 @@ ps_status build_tables(ps_batch* b) {
     B.nalpha = df{(float)(-alpha), (float)(-alpha - (double)(float)(-alpha))};
     B.singular = pn(d.bcx) && pn(d.bcy) && pn(d.bcz) && !B.shift;
     B.periodic_z = d.bcz == PS_BC_PERIODIC;
-    ps_plan_internal_tables(pl, &B.twx, &B.twy, &B.lamx, &B.lamy, &B.za, &B.zb, &B.zc, &B.dzf, &B.zlo,
-                            &B.zhi, &B.idx2, &B.idy2, &B.wsum_total, B.radx, B.rady, &B.nstx, &B.nsty);
+    ps_plan_internal_tables(pl, &B.tabx, &B.taby, &B.lamx, &B.lamy, &B.za, &B.zb, &B.zc, &B.dzf, &B.zlo,
+                            &B.zhi, &B.idx2, &B.idy2, &B.wsum_total);
     B.mx = d.nx / 2;
     B.my = d.ny / 2;
     const size_t N = (size_t)d.nx * d.ny * d.nz;
     // tiles: lines per task within 48 KB of shared memory, scaled by the tuned factor
-    auto lines_for = [&](int m, int axis) {
-      int L = 4 * b->scale;
-      const int cap = (int)(48 * 1024 / (2 * (size_t)(m + 1) * sizeof(cplx<float>)));
-      L = std::max(1, std::min(L, cap));
-      if (axis == 1) while (L > 1 && d.nx % L) --L;
-      return L;
+    auto lines_for = [&](int m) {
+      int lg = 2;
+      while ((1 << lg) < 4 * b->scale && lg < 10) ++lg;
+      while (lg > 0 && (batch_tile_smem(m, lg) > 48 * 1024 || (m << lg) > 32768)) --lg;
+      return lg;
     };
-    B.Lx = lines_for(B.mx, 0);
-    B.Ly = lines_for(B.my, 1);
+    B.lgx = lines_for(B.mx);
+    B.lgy = lines_for(B.my);
     B.res_chunk = 2048 * b->scale;
-    B.ntask[0] = (d.ny * d.nz + B.Lx - 1) / B.Lx;
-    B.ntask[1] = d.nz * (d.nx / B.Ly);
+    B.ntask[0] = (d.ny * d.nz + (1 << B.lgx) - 1) >> B.lgx;
+    B.ntask[1] = d.nz * ((d.nx + (1 << B.lgy) - 1) >> B.lgy);
     B.ntask[2] = (d.nx * d.ny + 255) / 256;
     B.ntask[3] = (int)((N + B.res_chunk - 1) / B.res_chunk);
-    smem = std::max(smem, 2 * (size_t)B.Lx * (B.mx + 1) * sizeof(cplx<float>));
-    smem = std::max(smem, 2 * (size_t)B.Ly * (B.my + 1) * sizeof(cplx<float>));
+    smem = std::max(smem, batch_tile_smem(B.mx, B.lgx));
+    smem = std::max(smem, batch_tile_smem(B.my, B.lgy));
     smem = std::max(smem, 2 * (size_t)d.nz * sizeof(float));
     // workspace slice: partials | w | scr | scr_u
     B.ws_off = ws_off;

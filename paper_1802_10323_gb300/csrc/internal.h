@@ -18,11 +18,34 @@ __host__ __device__ inline bool bc_iv(int bc) { return bc == BC_ND || bc == BC_D
 // kernels; longer ones in the shared-memory kernel, one line per CTA (two buffers
 // of n/2 + 1 complex values: 131 KB for an FP64 line of 8192)
 constexpr int kMaxN = 8192;
-constexpr int kMaxStages = 12;
+constexpr int kMaxStages = 6;   // of a generic line FFT (radices up to 9: m ≤ 4096 needs 4)
 extern thread_local char g_launch_diag[256];  // configuration of the last failed launch
 // Test hook (ps_inject_alloc_failures): true while injected device-allocation failures
 // remain; each call consumes one.
 bool take_injected_alloc_failure();
+
+// One Stockham stage of a generic line FFT of m points: radix r, nb = m/r butterflies,
+// ns the product of the earlier radices, tws = m/(ns·r), mg = ⌈2^32/ns⌉ (0 for ns = 1).
+struct FftStage {
+  int r, nb, ns, tws;
+  unsigned mg;
+};
+// A line's tables and FFT stages (device memory), made at plan creation. The split and
+// BC factors of xform_dev.cuh with their constants folded in, [0] backward, [1] forward:
+//   t0: k ≤ m/2: forward −(i/2)e^{−2πik/2m}, backward i·e^{+2πik/2m}/2m (FD: the forward one
+//       both ways); DCT-IV: e^{−iπk/n}, k < m;
+//   t1: NN, DD: q ≤ m: forward 2e^{−iπq/2n}, backward ½e^{+iπq/2n}; DCT-IV: k < m:
+//       e^{−iπ(4k+1)/4n} times 2 (forward) or 1/n (backward); else null.
+template <class T>
+struct LineTab {
+  const FftStage* stage;
+  int nstages;
+  unsigned mg_m, mg_h;      // reciprocals of m and n/2
+  T inv2m;                  // 1/(2m)
+  const cplx<T>* w;         // e^{−2πit/m}, t < m
+  const cplx<T>* t0[2];
+  const cplx<T>* t1[2];
+};
 
 // Arguments of one batch of line transforms (x or y).
 template <class T>
@@ -33,11 +56,9 @@ struct XformArgs {
   int axis;          // 0 = x (contiguous rows), 1 = y (strided by nx)
   int nx, ny, nz;
   int nlines;        // x: nz*ny rows
-  int L;             // lines per CTA (set by the launcher)
+  int lgL;           // log2 of the lines per tile (set by the launcher)
   int bc;
-  int nstages;
-  int radix[kMaxStages];
-  const cplx<T>* tw;        // e^{−2πi t/(8n)}, t = 0 … 8n−1
+  LineTab<T> tab;
   const T* plane_scale;     // per-z factor on load (fwd) / store (bwd), or null
   int accumulate;           // store: out = out + v
   const int* skip;          // if non-null and *skip != 0 the kernel returns at once
@@ -186,10 +207,9 @@ void set_plan_error(ps_plan* plan, const char* msg);
 
 // The FP32 tables of a plan (used by the batched solve).
 double ps_plan_internal_alpha(const ps_plan* p);  // the plan's Helmholtz shift (0: Poisson)
-void ps_plan_internal_tables(const ps_plan* p, const cplx<float>** twx, const cplx<float>** twy,
+void ps_plan_internal_tables(const ps_plan* p, LineTab<float>* tx, LineTab<float>* ty,
                              const float** lamx, const float** lamy, const float** za, const float** zb,
                              const float** zc, const float** dzf, const float2** zlo, const float2** zhi,
-                             df* idx2, df* idy2, double* wsum_total, int* radx, int* rady, int* nstx,
-                             int* nsty);
+                             df* idx2, df* idy2, double* wsum_total);
 
 }  // namespace ps

@@ -52,8 +52,9 @@ void cis(long t, long N, double* c, double* s) {
 }
 
 struct AxisTab {
-  int n = 0, m = 0, bc = 0, nstages = 0;
-  int radix[kMaxStages] = {0};
+  int n = 0, m = 0, bc = 0;
+  LineTab<double> g64{};  // generic line transforms (xform_dev.cuh)
+  LineTab<float> g32{}, gb{};  // (gb: the batched kernel's, radices up to 9)
   cplx<double>* tw64 = nullptr;
   cplx<float>* tw32 = nullptr;
   double* lam64 = nullptr;
@@ -68,12 +69,43 @@ bool size_ok(int n) {
   return m == 1;
 }
 
-int make_radix(int m, int* radix) {
-  int ns = 0;
-  while (m % 4 == 0) { radix[ns++] = 4; m /= 4; }
-  while (m % 2 == 0) { radix[ns++] = 2; m /= 2; }
-  while (m % 3 == 0) { radix[ns++] = 3; m /= 3; }
-  return ns;
+// ⌈2^32/d⌉, or 0 for d = 1 (div_mg, xform_dev.cuh)
+unsigned reciprocal(int d) { return d == 1 ? 0u : (unsigned)(((1ull << 32) + d - 1) / d); }
+
+// Stages of an m-point FFT: radices up to rmax, fewest stages first, then the smallest
+// sum of radices (the least arithmetic), in descending order (the first stage, the only
+// one without twiddles, takes the largest).
+void fft_stages(int m, int rmax, std::vector<FftStage>* out) {
+  static const int R[] = {16, 9, 8, 6, 4, 3, 2};
+  std::vector<int> best, cur;
+  auto worse = [&](const std::vector<int>& a, const std::vector<int>& b) {  // a no better than b
+    if (a.size() != b.size()) return a.size() > b.size();
+    int sa = 0, sb = 0;
+    for (int r : a) sa += r;
+    for (int r : b) sb += r;
+    return sa >= sb;
+  };
+  bool have = false;
+  auto dfs = [&](auto&& self, int rest, int first) -> void {
+    if (rest == 1) {
+      if (!have || !worse(cur, best)) best = cur;
+      have = true;
+      return;
+    }
+    if ((int)cur.size() == kMaxStages) return;
+    for (int i = first; i < 7; ++i)
+      if (R[i] <= rmax && rest % R[i] == 0) {
+        cur.push_back(R[i]);
+        self(self, rest / R[i], i);
+        cur.pop_back();
+      }
+  };
+  dfs(dfs, m, 0);
+  int ns = 1;
+  for (int r : best) {
+    out->push_back(FftStage{r, m / r, ns, m / (ns * r), reciprocal(ns)});
+    ns *= r;
+  }
 }
 
 // θ_q of Table 1 as a multiple of π/(4n): θ_q = π·j/(4n).
@@ -96,6 +128,89 @@ std::vector<double> eig_scaled(int bc, int n, double h) {
   }
   if (bc == BC_FD) lam[0] = -1.0 / (h * h);  // the wall face's own row −u_0/Δ²
   return lam;
+}
+
+// ---- tables of the generic line transforms (LineTab, internal.h) ----------------
+size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+int gen_m(int bc, int n) { return bc == BC_FD ? n : n / 2; }
+
+// entries of the complex tables: w, t0 backward and forward, t1 backward and forward
+size_t gen_entries(int bc, int n) {
+  const size_t m = gen_m(bc, n), h = m / 2 + 1;
+  if (bc_iv(bc)) return m + m + 2 * m;
+  if (bc == BC_NN || bc == BC_DD) return m + 2 * h + 2 * (m + 1);
+  return m + 2 * h;
+}
+size_t gen_table_bytes(int bc, int n) {
+  const size_t e = gen_entries(bc, n);
+  return al256(e * sizeof(cplx<double>)) + al256(e * sizeof(cplx<float>)) + 2 * al256(kMaxStages * sizeof(FftStage));
+}
+
+// tw: e^{−2πi t/(8n)}, t < 8n (every factor below is one of its entries, times a constant)
+template <class Take, class Put>
+void gen_tables(AxisTab& t, const std::vector<cplx<double>>& tw, Take&& take, Put&& hput) {
+  const int n = t.n, m = t.m, h = m / 2 + 1;
+  std::vector<cplx<double>> v;
+  size_t o_t0[2], o_t1[2] = {0, 0};
+  v.reserve(gen_entries(t.bc, n));
+  auto push = [&](int num, double fr, double fi) {  // (fr + i·fi)·e^{−2πi·num/16m}; 16m = 8n (FD: 16n)
+    const int i = t.bc == BC_FD ? num / 2 : num;
+    const double c = tw[i < 0 ? -i : i].x, s = i < 0 ? tw[-i].y : -tw[i].y;
+    v.push_back({fr * c + fi * s, fi * c - fr * s});
+  };
+  for (int i = 0; i < m; ++i) push(16 * i, 1.0, 0.0);
+  const bool iv = bc_iv(t.bc), two = t.bc == BC_NN || t.bc == BC_DD;
+  if (iv) {  // n = 2m: e^{−iπk/n} = e^{−2πi·4k/16m}, e^{−iπ(4k+1)/4n} = e^{−2πi(4k+1)/16m}
+    o_t0[0] = o_t0[1] = v.size();
+    for (int k = 0; k < m; ++k) push(4 * k, 1.0, 0.0);
+    o_t1[0] = v.size();
+    for (int k = 0; k < m; ++k) push(4 * k + 1, 1.0 / n, 0.0);
+    o_t1[1] = v.size();
+    for (int k = 0; k < m; ++k) push(4 * k + 1, 2.0, 0.0);
+  } else {
+    o_t0[0] = v.size();
+    for (int k = 0; k < h; ++k) {
+      if (t.bc == BC_FD) push(8 * k, 0.0, -0.5);
+      else push(-8 * k, 0.0, 1.0 / (2.0 * m));
+    }
+    o_t0[1] = v.size();
+    for (int k = 0; k < h; ++k) push(8 * k, 0.0, -0.5);
+    if (two) {  // e^{−iπq/2n} = e^{−2πi·2q/16m}
+      o_t1[0] = v.size();
+      for (int q = 0; q <= m; ++q) push(-2 * q, 0.5, 0.0);
+      o_t1[1] = v.size();
+      for (int q = 0; q <= m; ++q) push(2 * q, 2.0, 0.0);
+    }
+  }
+  std::vector<cplx<float>> v32;
+  for (const auto& z : v) v32.push_back({(float)z.x, (float)z.y});
+  cplx<double>* d64 = reinterpret_cast<cplx<double>*>(take(v.size() * sizeof(cplx<double>)));
+  cplx<float>* d32 = reinterpret_cast<cplx<float>*>(take(v.size() * sizeof(cplx<float>)));
+  hput(d64, v.data(), v.size() * sizeof(v[0]));
+  hput(d32, v32.data(), v32.size() * sizeof(v32[0]));
+  std::vector<FftStage> s16, s9;
+  fft_stages(m, 16, &s16);
+  fft_stages(m, 9, &s9);
+  FftStage* p16 = reinterpret_cast<FftStage*>(take(kMaxStages * sizeof(FftStage)));
+  FftStage* p9 = reinterpret_cast<FftStage*>(take(kMaxStages * sizeof(FftStage)));
+  hput(p16, s16.data(), s16.size() * sizeof(FftStage));
+  hput(p9, s9.data(), s9.size() * sizeof(FftStage));
+  auto fill = [&](auto& g, auto* d, const FftStage* st, int nst) {
+    g.stage = st;
+    g.nstages = nst;
+    g.mg_m = reciprocal(m);
+    g.mg_h = reciprocal(n / 2);
+    g.inv2m = (decltype(g.inv2m))(1.0 / (2.0 * m));
+    g.w = d;
+    for (int f = 0; f < 2; ++f) {
+      g.t0[f] = d + o_t0[f];
+      g.t1[f] = (iv || two) ? d + o_t1[f] : nullptr;
+    }
+  };
+  fill(t.g64, d64, p16, (int)s16.size());
+  fill(t.g32, d32, p16, (int)s16.size());
+  fill(t.gb, d32, p9, (int)s9.size());
 }
 
 void split_df(double d, float2* out) {
@@ -249,10 +364,8 @@ XformArgs<T> xargs(const ps_plan* p, int axis, const void* in, void* out, const 
   a.nz = p->nz;
   a.nlines = (axis == 0) ? p->ny * p->nz : p->nx * p->nz;
   a.bc = t.bc;
-  a.nstages = t.nstages;
-  for (int i = 0; i < kMaxStages; ++i) a.radix[i] = t.radix[i];
-  if constexpr (sizeof(T) == 8) a.tw = reinterpret_cast<const cplx<T>*>(t.tw64);
-  else a.tw = reinterpret_cast<const cplx<T>*>(t.tw32);
+  if constexpr (sizeof(T) == 8) a.tab = t.g64;
+  else a.tab = t.g32;
   a.plane_scale = scale;
   a.accumulate = accumulate;
   a.skip = skip;
@@ -723,13 +836,12 @@ bool take_injected_alloc_failure() {
 
 double ps_plan_internal_alpha(const ps_plan* p) { return p->alpha; }
 
-void ps_plan_internal_tables(const ps_plan* p, const cplx<float>** twx, const cplx<float>** twy,
+void ps_plan_internal_tables(const ps_plan* p, LineTab<float>* tx, LineTab<float>* ty,
                              const float** lamx, const float** lamy, const float** za, const float** zb,
                              const float** zc, const float** dzf, const float2** zlo, const float2** zhi,
-                             df* idx2, df* idy2, double* wsum_total, int* radx, int* rady, int* nstx,
-                             int* nsty) {
-  *twx = p->ax.tw32;
-  *twy = p->ay.tw32;
+                             df* idx2, df* idy2, double* wsum_total) {
+  *tx = p->ax.gb;
+  *ty = p->ay.gb;
   *lamx = p->ax.lam32;
   *lamy = p->ay.lam32;
   *za = p->za32;
@@ -741,12 +853,6 @@ void ps_plan_internal_tables(const ps_plan* p, const cplx<float>** twx, const cp
   *idx2 = p->idx2;
   *idy2 = p->idy2;
   *wsum_total = p->wsum * p->nx * p->ny;
-  for (int i = 0; i < kMaxStages; ++i) {
-    radx[i] = p->ax.radix[i];
-    rady[i] = p->ay.radix[i];
-  }
-  *nstx = p->ax.nstages;
-  *nsty = p->ay.nstages;
 }
 }  // namespace ps
 
@@ -905,6 +1011,7 @@ ps_status ps_plan_create_helmholtz(ps_plan** out, int nx, int ny, int nz, double
     const int n = ns[a];
     bytes += align256(8 * n * sizeof(cplx<double>)) + align256(8 * n * sizeof(cplx<float>));
     bytes += align256(n * sizeof(double)) + align256(n * sizeof(float));
+    bytes += gen_table_bytes(bcs[a], n);
   }
   bytes += 6 * align256(nz * sizeof(double)) + 6 * align256(nz * sizeof(float)) +
            2 * align256(nz * sizeof(float2)) + align256(3 * nz * sizeof(float2));
@@ -952,7 +1059,6 @@ ps_status ps_plan_create_helmholtz(ps_plan** out, int nx, int ny, int nz, double
     t.n = n;
     t.bc = bcs[a];
     t.m = t.bc == BC_FD ? n : n / 2;  // FD: the n-point FFT of the odd extension (xform_dev.cuh)
-    t.nstages = make_radix(t.m, t.radix);
     t.tw64 = reinterpret_cast<cplx<double>*>(take(8 * n * sizeof(cplx<double>)));
     t.tw32 = reinterpret_cast<cplx<float>*>(take(8 * n * sizeof(cplx<float>)));
     t.lam64 = reinterpret_cast<double*>(take(n * sizeof(double)));
@@ -971,6 +1077,7 @@ ps_status ps_plan_create_helmholtz(ps_plan** out, int nx, int ny, int nz, double
     hput(t.tw32, tw32.data(), tw32.size() * sizeof(tw32[0]));
     hput(t.lam64, lam.data(), n * sizeof(double));
     hput(t.lam32, lam32.data(), n * sizeof(float));
+    gen_tables(t, tw64, take, hput);
   }
   double** d64[6] = {&p->za64, &p->zb64, &p->zc64, &p->dzf64, &p->idzf64, &p->idzc64};
   float** d32[6] = {&p->za32, &p->zb32, &p->zc32, &p->dzf32, &p->idzf32, &p->idzc32};

@@ -1,8 +1,8 @@
 // xform_dev.cuh — device code of the generic line transforms (Table 2) along x or y.
 //
 // Every transform of length n (even) is reduced to one complex FFT of length
-// m = n/2 done in shared memory (Stockham, radix 4/2/3), with BC-specific
-// pre- and post-processing:
+// m = n/2 done in shared memory (Stockham, radices 16, 9, 8, 6, 4, 3, 2), with
+// BC-specific pre- and post-processing:
 //   P   (DFT, half-complex layout): z_p = a_2p + i a_2p+1, then the standard
 //        even/odd split X_k = E_k + e^{−2πik/n} O_k.
 //   NN  (DCT-II / DCT-III): Makhoul's reordering v_j = a_2j, v_{n−1−j} = a_2j+1,
@@ -17,362 +17,383 @@
 //        FFT of m = n complex points z_j = y_2j + i y_2j+1 and the real-DFT split
 //        Y_k = E_k + e^{−iπk/n} O_k, giving X_k = −Im(Y_k). DST-I is its own inverse
 //        up to 2n, so the backward transform is the same with the factor 1/(2n).
-// Backward transforms include Table 1's normalisation (1/n or 1/2n).
+// Backward transforms include Table 1's normalisation (1/n or 1/2n). Their inverse
+// FFT is the forward one with the two parts of every complex value traded.
 //
-// One CTA transforms L lines. x-lines are contiguous rows of the
-// [n_z][n_y][n_x] array; y-lines are strided by n_x and a CTA takes L
-// consecutive x columns of one z plane, so its global loads and stores are
-// coalesced across the L columns (the transposes of the pencil algorithm of
-// §3 become this strided tiling).
+// One CTA transforms a tile of L lines (x: L consecutive rows of the
+// [n_z][n_y][n_x] array; y: L consecutive x columns of one z plane, the last tile of
+// a plane partial when L does not divide n_x). The line lengths are run-time values
+// (any n/2 = 2^a·3^b); what keeps the index work small is the layout:
+//   * shared memory holds the tile as complex slots [slot][line] with the lanes of a
+//     half-warp (L = 16) on consecutive lines, so that every stage access is
+//     conflict-free whatever the stride of the slots, and the butterfly index and
+//     its twiddles are shared by those lanes (broadcast loads);
+//   * the reals go straight to the slot and part where the FFT wants them (the
+//     permutations of P, NN, DD and ND are such scatters), and the paired pre- and
+//     post-processing works in place: slot k ends as the two outputs of wavenumber k;
+//   * y lines are read and written as row segments of L values; x lines in pairs of
+//     values with the lanes along the line (the slots' row pitch L + 1 keeps those
+//     transposing accesses conflict-free);
+//   * the factors ½, 2 and 1/m of the split and of the normalisation sit in the
+//     plan's tables, and divisions by run-time lengths are multiplications by their
+//     reciprocals.
+// Bound by instruction issue (the index arithmetic of run-time lengths, 57–69 % issue
+// active in FP32), in FP64 by the FP64 pipe. Measured on 384×288×201 against the kernel this
+// one replaced (one row per line, radices 4, 2 and 3, twiddles at stride 16 from the plan's
+// 8n-entry table): FP32 x pass 300 → 97 µs forward, 344 → 99 µs backward, y passes
+// 247 → 113 and 230 → 105 µs; 192×96×65: 25–37 → 13–16 µs a pass.
 #pragma once
-#include "internal.h"
+#include "xform_units.cuh"
 
 namespace ps {
 
-template <class T, bool INV>
-__device__ __forceinline__ void bfly2(cplx<T>* v) {
-  cplx<T> a = v[0], b = v[1];
-  v[0] = cadd(a, b);
-  v[1] = csub(a, b);
-}
-
-template <class T, bool INV>
-__device__ __forceinline__ void bfly4(cplx<T>* v) {
-  cplx<T> t0 = cadd(v[0], v[2]), t1 = csub(v[0], v[2]);
-  cplx<T> t2 = cadd(v[1], v[3]), t3 = csub(v[1], v[3]);
-  t3 = INV ? mul_i(t3) : mul_mi(t3);
-  v[0] = cadd(t0, t2);
-  v[1] = cadd(t1, t3);
-  v[2] = csub(t0, t2);
-  v[3] = csub(t1, t3);
-}
-
-template <class T, bool INV>
-__device__ __forceinline__ void bfly3(cplx<T>* v) {
+template <class T>
+__device__ __forceinline__ void dft3(cplx<T>* v) {
   const T s3 = (T)0.86602540378443864676;  // sin(π/3)
-  cplx<T> t = cadd(v[1], v[2]);
-  cplx<T> d = csub(v[1], v[2]);
-  cplx<T> x0 = cadd(v[0], t);
-  cplx<T> u = {v[0].x - (T)0.5 * t.x, v[0].y - (T)0.5 * t.y};
-  cplx<T> w = INV ? mul_i(cscale(d, s3)) : mul_mi(cscale(d, s3));
-  v[0] = x0;
-  v[1] = cadd(u, w);
-  v[2] = csub(u, w);
+  const cplx<T> t = cadd(v[1], v[2]), d = csub(v[1], v[2]);
+  const cplx<T> u = {v[0].x - (T)0.5 * t.x, v[0].y - (T)0.5 * t.y};
+  v[0] = cadd(v[0], t);
+  v[1] = {u.x + s3 * d.y, u.y - s3 * d.x};
+  v[2] = {u.x - s3 * d.y, u.y + s3 * d.x};
 }
 
-// One Stockham stage of radix R over L lines of m points (row stride ld).
-// tw is the 8n-entry table e^{−2πi t/(8n)}; ω_m^x = tw[twm·x] with twm = 8n/m
-// (16 for the m = n/2 FFTs, 8 for the m = n FFT of a face-centred line).
-template <class T, int R, bool INV>
-__device__ __forceinline__ void stage(const cplx<T>* __restrict__ src, cplx<T>* __restrict__ dst,
-                                      int L, int m, int ld, int Ns, const cplx<T>* __restrict__ tw, int twm) {
-  const int nb = m / R;
-  const int tws = m / (Ns * R);
-  for (int idx = threadIdx.x; idx < L * nb; idx += blockDim.x) {
-    const int l = idx / nb;
-    const int j = idx - l * nb;
-    const int k = j % Ns;
-    const cplx<T>* s = src + l * ld;
-    cplx<T> v[R];
+// 6 = 2 × 3 by the prime-factor map: X[(3·k1 + 4·k2) mod 6] from x[(3·n1 + 2·n2) mod 6], no twiddles
+template <class T>
+__device__ __forceinline__ void dft6(cplx<T>* v) {
+  cplx<T> a[3] = {v[0], v[2], v[4]}, b[3] = {v[3], v[5], v[1]};
+  dft3(a);
+  dft3(b);
+  v[0] = cadd(a[0], b[0]);
+  v[3] = csub(a[0], b[0]);
+  v[4] = cadd(a[1], b[1]);
+  v[1] = csub(a[1], b[1]);
+  v[2] = cadd(a[2], b[2]);
+  v[5] = csub(a[2], b[2]);
+}
+
+// 9 = 3 × 3: X[k1 + 3k2] = Σ_{n2} W3^{n2·k2} W9^{n2·k1} Σ_{n1} x[n2 + 3n1] W3^{n1·k1}
+template <class T>
+__device__ __forceinline__ void dft9(cplx<T>* v) {
+  const cplx<T> w1 = {(T)0.76604444311897803520, (T)-0.64278760968653932632};   // e^{−2πi/9}
+  const cplx<T> w2 = {(T)0.17364817766693034885, (T)-0.98480775301220805937};   // e^{−4πi/9}
+  const cplx<T> w4 = {(T)-0.93969262078590838405, (T)-0.34202014332566873304};  // e^{−8πi/9}
+  cplx<T> a[3][3];
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[r] = s[j + r * nb];
-    if (Ns > 1) {
+  for (int q = 0; q < 3; ++q) {
 #pragma unroll
-      for (int r = 1; r < R; ++r) {
-        cplx<T> w = tw[twm * (r * k * tws)];
-        if (INV) w.y = -w.y;
-        v[r] = cmul(v[r], w);
-      }
-    }
-    if constexpr (R == 2) bfly2<T, INV>(v);
-    if constexpr (R == 3) bfly3<T, INV>(v);
-    if constexpr (R == 4) bfly4<T, INV>(v);
-    cplx<T>* d = dst + l * ld + (j / Ns) * Ns * R + k;
+    for (int r = 0; r < 3; ++r) a[q][r] = v[q + 3 * r];
+    dft3(a[q]);
+  }
+  a[1][1] = cmul(a[1][1], w1);
+  a[1][2] = cmul(a[1][2], w2);
+  a[2][1] = cmul(a[2][1], w2);
+  a[2][2] = cmul(a[2][2], w4);
 #pragma unroll
-    for (int r = 0; r < R; ++r) d[r * Ns] = v[r];
+  for (int k1 = 0; k1 < 3; ++k1) {
+    cplx<T> b[3] = {a[0][k1], a[1][k1], a[2][k1]};
+    dft3(b);
+#pragma unroll
+    for (int k2 = 0; k2 < 3; ++k2) v[k1 + 3 * k2] = b[k2];
   }
 }
 
-// Makhoul index map: position j of v ↔ position of a.
-__device__ __forceinline__ int mk_idx(int j, int n, int m) { return j < m ? 2 * j : 2 * n - 1 - 2 * j; }
+template <class T>
+__device__ __forceinline__ cplx<T> ldg_c(const cplx<T>* p) {  // a table entry (constant for the kernel)
+  if constexpr (sizeof(T) == 4) {
+    const float2 t = __ldg(reinterpret_cast<const float2*>(p));
+    return {t.x, t.y};
+  } else {
+    const double2 t = __ldg(reinterpret_cast<const double2*>(p));
+    return {t.x, t.y};
+  }
+}
 
-// Transforms line group `grp` (x: rows grp*L …; y: L columns of one z plane);
-// every thread of the CTA takes part; smem_raw holds 2·L·(m+1) complex values.
-template <class T, class TI, class TO, bool FWD>
+// ⌊i/d⌋ for 0 ≤ i < 2^16 from mg = ⌈2^32/d⌉ (d = 1: mg = 0)
+__device__ __forceinline__ int div_mg(int i, unsigned mg) { return mg ? (int)__umulhi((unsigned)i, mg) : i; }
+
+// One Stockham stage of radix R over the tile's lines. `pre`: a table to multiply the
+// stage's inputs with (first stage of the DCT-IV family), or null.
+template <class T, int R>
+__device__ __forceinline__ void gen_stage(const cplx<T>* src, cplx<T>* dst, int lgL, int ls, int m,
+                                          const FftStage& S, const cplx<T>* __restrict__ w,
+                                          const cplx<T>* __restrict__ pre) {
+  const int nb = S.nb, ns = S.ns, lm = (1 << lgL) - 1;
+  for (int idx = threadIdx.x; idx < (nb << lgL); idx += blockDim.x) {
+    const int l = idx & lm, j = idx >> lgL;
+    const cplx<T>* s = src + j * ls + l;
+    cplx<T> v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = s[r * nb * ls];
+    if (pre) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[r] = cmul(v[r], ldg_c(pre + j + r * nb));
+    }
+    const int q = div_mg(j, S.mg), k = j - q * ns;
+    if (ns > 1) {
+      const cplx<T>* wk = w + k * S.tws;
+#pragma unroll
+      for (int r = 1; r < R; ++r) v[r] = cmul(v[r], ldg_c(wk + (r - 1) * k * S.tws));
+    }
+    if constexpr (R == 3) dft3(v);
+    else if constexpr (R == 6) dft6(v);
+    else if constexpr (R == 9) dft9(v);
+    else col::dft<T, R, false>(v);
+    cplx<T>* d = dst + (q * ns * R + k) * ls + l;
+#pragma unroll
+    for (int r = 0; r < R; ++r) d[r * ns * ls] = v[r];
+  }
+}
+
+// A pair of consecutive values (e, e + 1), e even; al: the address is aligned to the pair
+template <class V>
+__device__ __forceinline__ void ld_pair(const V* p, bool al, V& a, V& b) {
+  if (al) {
+    const row::vec<V, 2> t = *reinterpret_cast<const row::vec<V, 2>*>(p);
+    a = t.v[0];
+    b = t.v[1];
+  } else {
+    a = p[0];
+    b = p[1];
+  }
+}
+template <class V>
+__device__ __forceinline__ void st_pair(V* p, bool al, V a, V b) {
+  if (al) {
+    row::vec<V, 2> t;
+    t.v[0] = a;
+    t.v[1] = b;
+    *reinterpret_cast<row::vec<V, 2>*>(p) = t;
+  } else {
+    p[0] = a;
+    p[1] = b;
+  }
+}
+
+// Where the line elements sit in the slots. Physical side (the field's values): the
+// elements (e0, e1) of slot p's two parts, and the signs of the DST ordering.
+struct SlotMap {
+  int n, m, bc;
+  __device__ __forceinline__ int mk(int j) const { return j < m ? 2 * j : 2 * n - 1 - 2 * j; }  // Makhoul (n = 2m)
+  __device__ __forceinline__ void phys(int p, int& e0, int& e1) const {
+    if (bc == BC_P) {
+      e0 = 2 * p;
+      e1 = 2 * p + 1;
+    } else if (bc == BC_ND) {
+      e0 = 2 * p;
+      e1 = n - 1 - 2 * p;
+    } else if (bc == BC_DN) {  // the reversed line: the two parts trade places
+      e0 = n - 1 - 2 * p;
+      e1 = 2 * p;
+    } else {
+      e0 = mk(2 * p);
+      e1 = mk(2 * p + 1);
+    }
+  }
+  // spectral side: the coefficients (q0, q1) of slot k's two parts
+  __device__ __forceinline__ void spec(int k, int& q0, int& q1) const {
+    if (bc == BC_P) {
+      q0 = k == 0 ? 0 : 2 * k - 1;
+      q1 = k == 0 ? n - 1 : 2 * k;
+    } else if (bc_iv(bc)) {
+      q0 = 2 * k;
+      q1 = n - 1 - 2 * k;
+    } else {
+      q0 = k;
+      q1 = k == 0 ? m : n - k;
+      if (bc == BC_DD) {
+        q0 = n - 1 - q0;
+        q1 = n - 1 - q1;
+      }
+    }
+  }
+  // the inverse maps for the pair (e, e + 1), e even: slot s and part c of each
+  __device__ __forceinline__ void phys_of(int e, int& s0, int& c0, int& s1, int& c1) const {
+    const int h = e >> 1;
+    if (bc == BC_P) {
+      s0 = s1 = h;
+      c0 = 0;
+      c1 = 1;
+    } else if (bc_iv(bc)) {
+      s0 = h;
+      s1 = m - 1 - h;
+      c0 = bc == BC_DN;
+      c1 = bc != BC_DN;
+    } else {
+      const int j1 = n - 1 - h;
+      s0 = h >> 1;
+      c0 = h & 1;
+      s1 = j1 >> 1;
+      c1 = j1 & 1;
+    }
+  }
+  __device__ __forceinline__ void spec_one(int e, int& s, int& c) const {
+    if (bc == BC_P) {
+      const int k = (e + 1) >> 1;
+      s = k == m ? 0 : k;
+      c = e == 0 ? 0 : (k == m ? 1 : !(e & 1));
+    } else if (bc_iv(bc)) {
+      c = e & 1;
+      s = c ? (n - 1 - e) >> 1 : e >> 1;
+    } else {
+      const int q = bc == BC_DD ? n - 1 - e : e;
+      c = q >= m;
+      s = q == m ? 0 : (c ? n - q : q);
+    }
+  }
+  __device__ __forceinline__ void spec_of(int e, int& s0, int& c0, int& s1, int& c1) const {
+    spec_one(e, s0, c0);
+    spec_one(e + 1, s1, c1);
+  }
+};
+
+// Transforms tile `grp`; every thread of the CTA takes part; smem_raw holds
+// 2·(m + 1)·(L + 1) complex values (L = 1: 2·(m + 1)).
+template <class T, class TI, class TO, bool FWD, int MAXR = 16>
 __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_raw) {
-  const int n = a.n, m = a.m, L = a.L, ld = m + 1, ldr = 2 * ld;
+  const LineTab<T>& tab = a.tab;
+  const cplx<T>* t0 = tab.t0[FWD];
+  const cplx<T>* t1 = tab.t1[FWD];
+  const int n = a.n, m = a.m, lgL = a.lgL, L = 1 << lgL, lm = L - 1, ls = L > 1 ? L + 1 : 1;
   cplx<T>* bufA = reinterpret_cast<cplx<T>*>(smem_raw);
-  cplx<T>* bufB = bufA + L * ld;
+  cplx<T>* bufB = bufA + (m + 1) * ls;
+  T* rA = reinterpret_cast<T*>(bufA);
   // no __restrict__: in and out may be the same array, and in the batched kernel
   // other CTAs rewrite it between tasks (the read-only cache path must not be used)
   const TI* in = static_cast<const TI*>(a.in);
   TO* out = static_cast<TO*>(a.out);
-  const cplx<T>* __restrict__ tw = a.tw;
-  const int nx = a.nx, ny = a.ny;
+  const int nx = a.nx, ny = a.ny, bc = a.bc;
+  const bool iv = bc_iv(bc), fd = bc == BC_FD;
+  const SlotMap map{n, m, bc};
+  const int tid = threadIdx.x, nt = blockDim.x;
 
-  // ---- line addressing -------------------------------------------------------
-  // x: line index ln = grp*L + l is the row (z*ny + y); element e at ln*n + e.
-  // y: grp = z*(nx/L) + xg; line l is column x = xg*L + l; element e at
-  //    z*ny*nx + e*nx + x.
-  const int gpz = nx / L;  // y only
-  const int zb = (a.axis == 1) ? grp / gpz : 0;
-  const int x0 = (a.axis == 1) ? (grp - zb * gpz) * L : 0;
-  const size_t ybase = (size_t)zb * ny * nx + x0;
-  const int nlines_here = (a.axis == 0) ? min(L, a.nlines - (int)grp * L) : L;
+  // ---- the tile: x: first element of row 0 of the group; y: column x0 of plane zb ----
+  const int gpz = a.axis == 1 ? (nx + L - 1) >> lgL : 1;
+  const int zb = a.axis == 1 ? grp / gpz : 0;
+  const int x0 = a.axis == 1 ? (grp - zb * gpz) << lgL : 0;
+  const size_t base = a.axis == 0 ? (size_t)grp * L * n : (size_t)zb * ny * nx + x0;
+  const int live = a.axis == 0 ? min(L, a.nlines - grp * L) : min(L, nx - x0);
+  auto scale_of = [&](int l) { return a.plane_scale[a.axis == 0 ? (grp * L + l) / ny : zb]; };
+  const bool fscale = FWD && a.plane_scale, bscale = !FWD && a.plane_scale;
 
-  // ---- 1. load (into bufB as reals) -------------------------------------------
-  T* rB = reinterpret_cast<T*>(bufB);
-  for (int idx = threadIdx.x; idx < L * n; idx += blockDim.x) {
-    int l, e;
-    size_t g;
-    int z;
-    if (a.axis == 0) {
-      l = idx / n;
-      e = idx - l * n;
-      if (l >= nlines_here) continue;
-      size_t ln = (size_t)grp * L + l;
-      g = ln * n + e;
-      z = (int)(ln / ny);
-    } else {
-      e = idx / L;
-      l = idx - e * L;
-      g = ybase + (size_t)e * nx + l;
-      z = zb;
-    }
-    T v = ld_cvt<T, TI>::f(in[g]);
-    if (FWD && a.plane_scale) v *= a.plane_scale[z];
-    rB[l * ldr + e] = v;
-  }
-  __syncthreads();
-
-  // ---- 2. pre-processing: reals (bufB) -> m complex points (bufA) ---------------
-  const int bc = a.bc;
-  if (bc == BC_FD) {  // both directions: z_j = (y_2j, y_2j+1) of the odd extension (m = n)
-    for (int idx = threadIdx.x; idx < L * m; idx += blockDim.x) {
-      const int l = idx / m, j = idx - l * m;
-      const T* x = rB + l * ldr;
-      auto y = [&](int t) -> T { return (t == 0 || t == n) ? (T)0 : (t < n ? x[t] : -x[2 * n - t]); };
-      bufA[l * ld + j] = cplx<T>{y(2 * j), y(2 * j + 1)};
-      if (j == 0) bufA[l * ld + m] = cplx<T>{x[0], (T)0};  // the wall entry, in the slot no stage writes
-    }
-  } else if (FWD) {
-    for (int idx = threadIdx.x; idx < L * m; idx += blockDim.x) {
-      const int l = idx / m, p = idx - l * m;
-      const T* x = rB + l * ldr;
-      cplx<T> z;
-      if (bc == BC_P) {
-        z = {x[2 * p], x[2 * p + 1]};
-      } else if (bc == BC_NN || bc == BC_DD) {
-        const int j0 = 2 * p, j1 = 2 * p + 1;
-        T v0 = x[mk_idx(j0, n, m)], v1 = x[mk_idx(j1, n, m)];
-        if (bc == BC_DD) {  // (−1)^index: odd a-indices come from j ≥ m
-          if (j0 >= m) v0 = -v0;
-          if (j1 >= m) v1 = -v1;
-        }
-        z = {v0, v1};
-      } else {  // ND (DN: the reversed line, the two reals swap)
-        const T e0 = x[2 * p], e1 = x[n - 1 - 2 * p];
-        z = cmul(bc == BC_DN ? cplx<T>{e1, e0} : cplx<T>{e0, e1}, tw[4 * p]);
+  // ---- 1. load into the slots of bufA ----
+  if (fd) {
+    // z_j = (y_2j, y_2j+1) of the odd extension, both directions (m = n); the wall
+    // entry is kept in slot m, which no stage writes
+    auto val = [&](int l, int t) -> T {
+      if (t == 0 || t == n) return (T)0;
+      const int e = t < n ? t : 2 * n - t;
+      const T v = ld_cvt<T, TI>::f(a.axis == 0 ? in[base + (size_t)l * n + e] : in[base + (size_t)e * nx + l]);
+      return t < n ? v : -v;
+    };
+    for (int idx = tid; idx < (m << lgL); idx += nt) {
+      const int l = a.axis == 0 ? div_mg(idx, tab.mg_m) : (idx & lm);
+      const int j = a.axis == 0 ? idx - l * m : idx >> lgL;
+      if (l >= live) continue;
+      const T sc = fscale ? scale_of(l) : (T)1;
+      bufA[j * ls + l] = cplx<T>{val(l, 2 * j) * sc, val(l, 2 * j + 1) * sc};
+      if (j == 0) {
+        const T w = ld_cvt<T, TI>::f(a.axis == 0 ? in[base + (size_t)l * n] : in[base + l]);
+        bufA[m * ls + l] = cplx<T>{w * sc, (T)0};
       }
-      bufA[l * ld + p] = z;
+    }
+  } else if (a.axis == 0) {
+    const bool al = !((uintptr_t)in & (2 * sizeof(TI) - 1));
+    const T sg = (FWD && bc == BC_DD) ? (T)-1 : (T)1;  // DST ordering: the odd elements change sign
+    for (int idx = tid; idx < live * m; idx += nt) {
+      const int l = div_mg(idx, tab.mg_m), e = 2 * (idx - l * m);
+      TI u0, u1;
+      ld_pair(in + base + (size_t)l * n + e, al, u0, u1);
+      T v0 = ld_cvt<T, TI>::f(u0), v1 = ld_cvt<T, TI>::f(u1);
+      if (fscale) {
+        const T sc = scale_of(l);
+        v0 *= sc;
+        v1 *= sc;
+      }
+      int s0, c0, s1, c1;
+      if (FWD) map.phys_of(e, s0, c0, s1, c1);
+      else map.spec_of(e, s0, c0, s1, c1);
+      rA[2 * (s0 * ls + l) + c0] = v0;
+      rA[2 * (s1 * ls + l) + c1] = sg * v1;
     }
   } else {
-    const int np = bc_iv(bc) ? m : (m / 2 + 1);
-    for (int idx = threadIdx.x; idx < L * np; idx += blockDim.x) {
-      const int l = idx / np, k = idx - l * np;
-      const T* X = rB + l * ldr;
-      cplx<T>* Z = bufA + l * ld;
-      if (bc_iv(bc)) {
-        Z[k] = cmul(cplx<T>{X[2 * k], X[n - 1 - 2 * k]}, tw[4 * k]);
-        continue;
+    const T sc = fscale ? a.plane_scale[zb] : (T)1;
+#pragma unroll 4
+    for (int idx = tid; idx < (m << lgL); idx += nt) {
+      const int l = idx & lm, p = idx >> lgL;
+      if (l >= live) continue;
+      int e0, e1;
+      if (FWD) map.phys(p, e0, e1);
+      else map.spec(p, e0, e1);
+      T v0 = ld_cvt<T, TI>::f(in[base + (size_t)(e0 * nx) + l]), v1 = ld_cvt<T, TI>::f(in[base + (size_t)(e1 * nx) + l]);
+      if (FWD) {
+        if (bc == BC_DD) {
+          if (e0 & 1) v0 = -v0;
+          if (e1 & 1) v1 = -v1;
+        }
+        v0 *= sc;
+        v1 *= sc;
       }
-      // spectrum V_k and V_{m−k} of the real sequence whose half-length FFT we invert
-      cplx<T> Vk, Vmk;
-      if (bc == BC_P) {
-        if (k == 0) {
-          Vk = {X[0], (T)0};
-          Vmk = {X[n - 1], (T)0};
-        } else {
-          Vk = {X[2 * k - 1], -X[2 * k]};
-          Vmk = {X[2 * (m - k) - 1], -X[2 * (m - k)]};
-        }
-      } else {
-        // DCT-III via Makhoul: V_q = e^{+iπq/2n} (X_q − i X_{n−q}) / 2, X_n = 0.
-        // DST-III: the same on Y_q = X_{n−1−q}.
-        const bool rev = (bc == BC_DD);
-#define XQ(q) ((q) >= n ? (T)0 : X[rev ? (n - 1 - (q)) : (q)])
-        {
-          const int q = k;
-          cplx<T> w = tw[2 * q];
-          w.y = -w.y;
-          cplx<T> s = {XQ(q), -XQ(n - q)};
-          Vk = cscale(cmul(w, s), (T)0.5);
-        }
-        {
-          const int q = m - k;
-          cplx<T> w = tw[2 * q];
-          w.y = -w.y;
-          cplx<T> s = {XQ(q), -XQ(n - q)};
-          Vmk = cscale(cmul(w, s), (T)0.5);
-        }
-#undef XQ
-      }
-      // E_k = (V_k + conj V_{m−k})/2, O_k = (V_k − conj V_{m−k}) e^{+2πik/n}/2
-      cplx<T> E = cscale(cadd(Vk, conj_(Vmk)), (T)0.5);
-      cplx<T> wn = tw[8 * k];
-      wn.y = -wn.y;
-      cplx<T> O = cscale(cmul(csub(Vk, conj_(Vmk)), wn), (T)0.5);
-      Z[k] = cadd(E, mul_i(O));
-      if (k != 0 && 2 * k != m) Z[m - k] = cadd(conj_(E), mul_i(conj_(O)));
+      bufA[p * ls + l] = cplx<T>{v0, v1};
     }
   }
   __syncthreads();
 
-  // ---- 3. complex FFT of length m (forward e^{−2πi/m}; backward e^{+2πi/m}, except
-  //         DCT-IV, which is its own inverse and uses the forward FFT both ways) ----------
+  // ---- 2. backward P, NN, DD: the pairs (k, m−k), in place, the parts traded for the
+  //         inverse FFT: Z_k = (V_k + conj V_{m−k})/2m + pb_k·(V_k − conj V_{m−k}),
+  //         pb_k = i·e^{+2πik/n}/2m; NN, DD: V_q = xb_q·(X_q − i X_{n−q}), xb_q = ½e^{+iπq/2n} ----
+  if (!FWD && !iv && !fd) {
+    const int np = m / 2 + 1;
+    const T s = tab.inv2m;
+    for (int idx = tid; idx < (np << lgL); idx += nt) {
+      const int l = idx & lm, k = idx >> lgL;
+      cplx<T>* A = bufA + k * ls + l;
+      cplx<T>* B = bufA + (k == 0 ? 0 : m - k) * ls + l;
+      const cplx<T> x = *A, y = *B;
+      cplx<T> V, W;
+      if (bc == BC_P) {
+        V = k == 0 ? cplx<T>{x.x, (T)0} : cplx<T>{x.x, -x.y};
+        W = k == 0 ? cplx<T>{x.y, (T)0} : cplx<T>{y.x, -y.y};
+      } else {
+        V = cmul(ldg_c(t1 + k), k == 0 ? cplx<T>{x.x, (T)0} : cplx<T>{x.x, -x.y});
+        W = cmul(ldg_c(t1 + m - k), k == 0 ? cplx<T>{x.y, -x.y} : cplx<T>{y.x, -y.y});
+      }
+      const cplx<T> Sm = cadd(V, conj_(W)), D = cmul(ldg_c(t0 + k), csub(V, conj_(W)));
+      const cplx<T> Zk = {s * Sm.x + D.x, s * Sm.y + D.y}, Zm = {s * Sm.x - D.x, D.y - s * Sm.y};
+      *A = {Zk.y, Zk.x};
+      if (k != 0 && 2 * k != m) *B = {Zm.y, Zm.x};
+    }
+    __syncthreads();
+  }
+
+  // ---- 3. the FFT ----
   cplx<T>* src = bufA;
   cplx<T>* dst = bufB;
-  {
-    const bool inv = !FWD && !bc_iv(bc) && bc != BC_FD;
-    const int twm = (8 * n) / m;
-    int Ns = 1;
-    for (int s = 0; s < a.nstages; ++s) {
-      const int R = a.radix[s];
-      if (inv) {
-        if (R == 4) stage<T, 4, true>(src, dst, L, m, ld, Ns, tw, twm);
-        else if (R == 2) stage<T, 2, true>(src, dst, L, m, ld, Ns, tw, twm);
-        else stage<T, 3, true>(src, dst, L, m, ld, Ns, tw, twm);
-      } else {
-        if (R == 4) stage<T, 4, false>(src, dst, L, m, ld, Ns, tw, twm);
-        else if (R == 2) stage<T, 2, false>(src, dst, L, m, ld, Ns, tw, twm);
-        else stage<T, 3, false>(src, dst, L, m, ld, Ns, tw, twm);
-      }
-      __syncthreads();
-      cplx<T>* t = src;
-      src = dst;
-      dst = t;
-      Ns *= R;
+  for (int st = 0; st < tab.nstages; ++st) {
+    const FftStage& S = tab.stage[st];
+    const cplx<T>* pre = (iv && st == 0) ? t0 : nullptr;
+    switch (S.r) {
+      case 16: if constexpr (MAXR >= 16) gen_stage<T, 16>(src, dst, lgL, ls, m, S, tab.w, pre); break;
+      case 9: gen_stage<T, 9>(src, dst, lgL, ls, m, S, tab.w, pre); break;
+      case 8: gen_stage<T, 8>(src, dst, lgL, ls, m, S, tab.w, pre); break;
+      case 6: gen_stage<T, 6>(src, dst, lgL, ls, m, S, tab.w, pre); break;
+      case 4: gen_stage<T, 4>(src, dst, lgL, ls, m, S, tab.w, pre); break;
+      case 3: gen_stage<T, 3>(src, dst, lgL, ls, m, S, tab.w, pre); break;
+      default: gen_stage<T, 2>(src, dst, lgL, ls, m, S, tab.w, pre); break;
     }
+    __syncthreads();
+    cplx<T>* t = src;
+    src = dst;
+    dst = t;
   }
-  // result in src; dst is free for the real output
-  T* rO = reinterpret_cast<T*>(dst);
-
-  // ---- 4. post-processing: m complex points -> n reals --------------------------
-  if (bc == BC_FD) {  // X_k = −Im(Y_k), k = 1 … n−1 (× 1/2n backward); the wall entry copied
-    const T sc = FWD ? (T)1 : (T)1 / (T)(2 * n);
-    for (int idx = threadIdx.x; idx < L * n; idx += blockDim.x) {
-      const int l = idx / n, k = idx - l * n;
-      const cplx<T>* Z = src + l * ld;
-      T* o = rO + l * ldr;
-      if (k == 0) {  // the wall entry (saved beside the FFT data by the pre-processing)
-        o[0] = bufA[l * ld + m].x;
-        continue;
-      }
-      const cplx<T> Zk = Z[k], Zmk = Z[m - k];
-      const cplx<T> E = cscale(cadd(Zk, conj_(Zmk)), (T)0.5);
-      const cplx<T> O = cscale(mul_mi(csub(Zk, conj_(Zmk))), (T)0.5);
-      const cplx<T> Y = cadd(E, cmul(tw[4 * k], O));
-      o[k] = -Y.y * sc;
-    }
-  } else if (FWD) {
-    const int np = bc_iv(bc) ? m : (m / 2 + 1);
-    for (int idx = threadIdx.x; idx < L * np; idx += blockDim.x) {
-      const int l = idx / np, k = idx - l * np;
-      const cplx<T>* Z = src + l * ld;
-      T* o = rO + l * ldr;
-      if (bc_iv(bc)) {
-        cplx<T> c = cmul(tw[4 * k + 1], Z[k]);
-        o[2 * k] = (T)2 * c.x;
-        o[n - 1 - 2 * k] = (T)-2 * c.y;
-        continue;
-      }
-      // real DFT of the packed sequence: V_k = A + B, V_{m−k} = conj(A − B)
-      cplx<T> Zk = Z[k], Zmk = Z[k == 0 ? 0 : m - k];
-      cplx<T> E = cscale(cadd(Zk, conj_(Zmk)), (T)0.5);
-      cplx<T> O = cscale(mul_mi(csub(Zk, conj_(Zmk))), (T)0.5);
-      cplx<T> B = cmul(tw[8 * k], O);
-      cplx<T> Vk = cadd(E, B);
-      cplx<T> Vmk = conj_(csub(E, B));  // for k = 0 this is V_m
-      if (bc == BC_P) {
-        if (k == 0) {
-          o[0] = Vk.x;
-          o[n - 1] = Vmk.x;
-        } else {
-          o[2 * k - 1] = Vk.x;
-          o[2 * k] = -Vk.y;
-          if (2 * k != m) {
-            o[2 * (m - k) - 1] = Vmk.x;
-            o[2 * (m - k)] = -Vmk.y;
-          }
-        }
-      } else {
-        const bool rev = (bc == BC_DD);
-#define OUT(q, val) o[rev ? (n - 1 - (q)) : (q)] = (val)
-        if (k == 0) {
-          OUT(0, (T)2 * Vk.x);
-          OUT(m, (T)1.41421356237309504880 * Vmk.x);
-        } else {
-          cplx<T> c = cmul(tw[2 * k], Vk);
-          OUT(k, (T)2 * c.x);
-          OUT(n - k, (T)-2 * c.y);
-          if (2 * k != m) {
-            cplx<T> c2 = cmul(tw[2 * (m - k)], Vmk);
-            OUT(m - k, (T)2 * c2.x);
-            OUT(m + k, (T)-2 * c2.y);
-          }
-        }
-#undef OUT
-      }
-    }
-  } else {
-    const T inv_m = (T)1 / (T)m;
-    for (int idx = threadIdx.x; idx < L * m; idx += blockDim.x) {
-      const int l = idx / m, k = idx - l * m;
-      const cplx<T>* Z = src + l * ld;
-      T* o = rO + l * ldr;
-      if (bc_iv(bc)) {
-        const T s = (T)1 / (T)n;  // 2·(1/2n)
-        cplx<T> c = cmul(tw[4 * k + 1], Z[k]);
-        const T A = s * c.x, B = -s * c.y;  // DN: the two outputs trade places
-        o[2 * k] = (bc == BC_DN) ? B : A;
-        o[n - 1 - 2 * k] = (bc == BC_DN) ? A : B;
-      } else if (bc == BC_P) {
-        o[2 * k] = Z[k].x * inv_m;
-        o[2 * k + 1] = Z[k].y * inv_m;
-      } else {
-        const int i0 = mk_idx(2 * k, n, m), i1 = mk_idx(2 * k + 1, n, m);
-        T v0 = Z[k].x * inv_m, v1 = Z[k].y * inv_m;
-        if (bc == BC_DD) {
-          if (i0 & 1) v0 = -v0;
-          if (i1 & 1) v1 = -v1;
-        }
-        o[i0] = v0;
-        o[i1] = v1;
-      }
-    }
+  if (iv && tab.nstages == 0) {  // n = 2: the pre-factor of the one point
+    for (int l = tid; l < L; l += nt) src[l] = cmul(src[l], ldg_c(t0));
+    __syncthreads();
   }
-  __syncthreads();
 
-  // ---- 5. store ----------------------------------------------------------------------
+  // ---- 4. post-processing in place (y, forward and DCT-IV: straight to the rows) ----
+  T* rS = reinterpret_cast<T*>(src);
   T tmax = (T)0;  // max |new value| before widening (a 64-bit integer max would use the FP64 pipe)
-  for (int idx = threadIdx.x; idx < L * n; idx += blockDim.x) {
-    int l, e, z;
-    size_t g;
-    if (a.axis == 0) {
-      l = idx / n;
-      e = idx - l * n;
-      if (l >= nlines_here) continue;
-      size_t ln = (size_t)grp * L + l;
-      g = ln * n + e;
-      z = (int)(ln / ny);
-    } else {
-      e = idx / L;
-      l = idx - e * L;
-      g = ybase + (size_t)e * nx + l;
-      z = zb;
-    }
-    T v = rO[l * ldr + e];
-    if (!FWD && a.plane_scale) v *= a.plane_scale[z];
+  auto emit = [&](size_t g, T v) {  // one output value
     const TO x = st_cvt<TO, T>::f(v);
     if constexpr (sizeof(TO) == 8) {
       if (out) {
@@ -383,16 +404,145 @@ __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_
           out[g] = a.accumulate ? out[g] + x : x;
         }
       }
-      tmax = fmax(tmax, fabs(v));
-      if constexpr (sizeof(T) == 4)
+      if constexpr (sizeof(T) == 4) {
+        tmax = fmaxf(tmax, fabsf(v));
         if (a.out2) a.out2[g] = v;
+      }
     } else {
       out[g] = a.accumulate ? out[g] + x : x;
     }
+  };
+  const T yscale = (a.axis == 1 && bscale) ? a.plane_scale[zb] : (T)1;
+  // the two values of slot k: kept in the slot (x), or written to their rows (y)
+  auto put = [&](int k, int l, T v0, T v1) {
+    if (a.axis == 0) {
+      src[k * ls + l] = cplx<T>{v0, v1};
+    } else if (l < live) {
+      int e0, e1;
+      if (FWD) map.spec(k, e0, e1);
+      else map.phys(k, e0, e1);
+      emit(base + (size_t)(e0 * nx) + l, FWD ? v0 : v0 * yscale);
+      emit(base + (size_t)(e1 * nx) + l, FWD ? v1 : v1 * yscale);
+    }
+  };
+  if (fd) {  // X_k = −Im(Y_k), k = 1 … n−1 (× 1/2n backward), into part 0 of slot k
+    const T sc = FWD ? (T)1 : tab.inv2m;
+    for (int idx = tid; idx < ((m / 2 + 1) << lgL); idx += nt) {
+      const int l = idx & lm, k = idx >> lgL;
+      const cplx<T> Zk = src[k * ls + l], Zm = src[(k == 0 ? 0 : m - k) * ls + l];
+      const cplx<T> Sm = cadd(Zk, conj_(Zm)), D = cmul(ldg_c(t0 + k), csub(Zk, conj_(Zm)));
+      if (k == 0) {
+        rS[2 * l] = bufA[m * ls + l].x;
+      } else {
+        rS[2 * (k * ls + l)] = -((T)0.5 * Sm.y + D.y) * sc;
+        if (2 * k != m) rS[2 * ((m - k) * ls + l)] = ((T)0.5 * Sm.y - D.y) * sc;
+      }
+    }
+    __syncthreads();
+  } else if (iv) {  // c_k = t_k·U_k, t_k = 2e^{−iπ(4k+1)/4n} (backward: /2n); outputs Re, −Im
+    for (int idx = tid; idx < (m << lgL); idx += nt) {
+      const int l = idx & lm, k = idx >> lgL;
+      const cplx<T> c = cmul(ldg_c(t1 + k), src[k * ls + l]);
+      put(k, l, c.x, -c.y);
+    }
+    if (a.axis == 0) __syncthreads();
+  } else if (FWD) {
+    // real DFT of the packed sequence: V_k = (Z_k + conj Z_{m−k})/2 + pf_k·(Z_k − conj Z_{m−k}),
+    // pf_k = −(i/2)e^{−2πik/n}; NN, DD: X_q = Re(xf_q V_q), X_{n−q} = −Im, xf_q = 2e^{−iπq/2n}
+    for (int idx = tid; idx < ((m / 2 + 1) << lgL); idx += nt) {
+      const int l = idx & lm, k = idx >> lgL;
+      const cplx<T> Zk = src[k * ls + l], Zm = src[(k == 0 ? 0 : m - k) * ls + l];
+      const cplx<T> Sm = cadd(Zk, conj_(Zm)), D = cmul(ldg_c(t0 + k), csub(Zk, conj_(Zm)));
+      const cplx<T> V = {(T)0.5 * Sm.x + D.x, (T)0.5 * Sm.y + D.y};
+      const cplx<T> W = {(T)0.5 * Sm.x - D.x, D.y - (T)0.5 * Sm.y};  // V_{m−k}
+      if (bc == BC_P) {
+        if (k == 0) put(0, l, V.x, W.x);
+        else {
+          put(k, l, V.x, -V.y);
+          if (2 * k != m) put(m - k, l, W.x, -W.y);
+        }
+      } else if (k == 0) {
+        put(0, l, (T)2 * V.x, (T)1.41421356237309504880 * W.x);
+      } else {
+        const cplx<T> c1 = cmul(ldg_c(t1 + k), V);
+        put(k, l, c1.x, -c1.y);
+        if (2 * k != m) {
+          const cplx<T> c2 = cmul(ldg_c(t1 + m - k), W);
+          put(m - k, l, c2.x, -c2.y);
+        }
+      }
+    }
+    if (a.axis == 0) __syncthreads();
   }
-  if constexpr (sizeof(TO) == 8) {
+
+  // ---- 5. store ----
+  // backward P, NN, DD: the FFT's parts are still traded (part c of a slot is 1 − c)
+  const int sw = (!FWD && !iv && !fd) ? 1 : 0;
+  if (a.axis == 0) {
+    const T sg = (!FWD && bc == BC_DD) ? (T)-1 : (T)1;
+    const bool al = !((((uintptr_t)out) & (2 * sizeof(TO) - 1)) | (((uintptr_t)a.out2 | (uintptr_t)a.base32) & 7));
+    for (int idx = tid; idx < live * (n >> 1); idx += nt) {
+      const int l = div_mg(idx, tab.mg_h), e = 2 * (idx - l * (n >> 1));
+      int s0, c0, s1, c1;
+      if (fd) {
+        s0 = e;
+        s1 = e + 1;
+        c0 = c1 = 0;
+      } else if (FWD) {
+        map.spec_of(e, s0, c0, s1, c1);
+      } else {
+        map.phys_of(e, s0, c0, s1, c1);
+      }
+      T v0 = rS[2 * (s0 * ls + l) + (c0 ^ sw)], v1 = sg * rS[2 * (s1 * ls + l) + (c1 ^ sw)];
+      if (bscale) {
+        const T sc = scale_of(l);
+        v0 *= sc;
+        v1 *= sc;
+      }
+      const size_t g = base + (size_t)l * n + e;
+      if constexpr (sizeof(TO) == 8 && sizeof(T) == 4) {
+        if (out) {
+          double b0 = 0.0, b1 = 0.0;
+          const double w0 = widen_f32(v0), w1 = widen_f32(v1);
+          if (a.base32) {
+            float f0, f1;
+            ld_pair(a.base32 + g, al, f0, f1);
+            b0 = widen_f32(f0);
+            b1 = widen_f32(f1);
+          } else if (a.accumulate) {
+            ld_pair(out + g, al, b0, b1);
+          }
+          const bool add = a.base32 || a.accumulate;
+          st_pair(out + g, al, add ? b0 + w0 : w0, add ? b1 + w1 : w1);
+        }
+        tmax = fmaxf(tmax, fmaxf(fabsf(v0), fabsf(v1)));
+        if (a.out2) st_pair(a.out2 + g, al, v0, v1);
+      } else {
+        TO b0 = (TO)0, b1 = (TO)0;
+        if (a.accumulate) ld_pair(out + g, al, b0, b1);
+        st_pair(out + g, al, a.accumulate ? b0 + v0 : v0, a.accumulate ? b1 + v1 : v1);
+      }
+    }
+  } else if (fd) {
+    for (int idx = tid; idx < (n << lgL); idx += nt) {
+      const int l = idx & lm, e = idx >> lgL;
+      if (l < live) emit(base + (size_t)(e * nx) + l, rS[2 * (e * ls + l)] * yscale);
+    }
+  } else if (!FWD && !iv) {
+    for (int idx = tid; idx < (m << lgL); idx += nt) {
+      const int l = idx & lm, p = idx >> lgL;
+      if (l >= live) continue;
+      const cplx<T> z = src[p * ls + l];
+      int e0, e1;
+      map.phys(p, e0, e1);
+      const T v0 = (bc == BC_DD && (e0 & 1)) ? -z.y : z.y, v1 = (bc == BC_DD && (e1 & 1)) ? -z.x : z.x;
+      emit(base + (size_t)(e0 * nx) + l, v0 * yscale);
+      emit(base + (size_t)(e1 * nx) + l, v1 * yscale);
+    }
+  }
+  if constexpr (sizeof(TO) == 8 && sizeof(T) == 4) {
     if (a.amax) {
-      for (int o = 16; o > 0; o >>= 1) tmax = fmax(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+      for (int o = 16; o > 0; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
       const unsigned long long amax = (unsigned long long)__double_as_longlong(st_cvt<double, T>::f(tmax));
       if ((threadIdx.x & 31) == 0 && amax) atomicMax(a.amax, amax);
     }
