@@ -3,7 +3,7 @@
 // Every grid is its own problem of §2.1 (sizes, spacings, z faces and BC pairs
 // per grid) solved in FP32 with FP64 iterative refinement. The work of all
 // grids is cut into tasks (grid, stage, tile): x/y line groups of the
-// transforms (Table 2), blocks of z columns (Eq. 5), the singular column,
+// transforms (Table 2), blocks of z columns (Eq. 5; the singular column by itself),
 // residual tiles and the per-grid convergence test. A task table ordered by
 // stage (then grid, then tile) is walked by one persistent kernel whose CTAs
 // take the next task from a global counter. A task may start once every task of
@@ -33,7 +33,7 @@
 
 namespace ps {
 
-enum BStage { BS_XF64 = 0, BS_XF, BS_YF, BS_Z, BS_ZS, BS_YB, BS_XBST, BS_XBACC, BS_RES, BS_CHK, BS_FIN };
+enum BStage { BS_XF64 = 0, BS_XF, BS_YF, BS_Z, BS_YB, BS_XBST, BS_XBACC, BS_RES, BS_CHK, BS_FIN };
 
 struct BGrid {
   int nx, ny, nz, bcx, bcy, bcz, singular, periodic_z;
@@ -42,7 +42,9 @@ struct BGrid {
   int res_chunk;           // points per residual task
   int ntask[4];            // x tasks, y tasks, z tasks, residual tasks
   LineTab<float> tabx, taby;
-  const float *lamx, *lamy, *za, *zb, *zc, *dzf;
+  const float *lamx, *lamy, *za, *zg, *zc, *dzf;
+  const double* dzf64;
+  const float2* zdf;
   const float2 *zlo, *zhi;
   df idx2, idy2;
   int shift;               // Helmholtz grid: the residual row also holds −α·Φ
@@ -102,7 +104,8 @@ __device__ ZArgs<float> bz_args(const BGrid& G, char* ws) {
   z.scr_u = G.periodic_z ? reinterpret_cast<float*>(ws + G.ws_off + G.off_scru) : nullptr;
   z.nx = G.nx; z.ny = G.ny; z.nz = G.nz;
   z.lamx = G.lamx; z.lamy = G.lamy;
-  z.za = G.za; z.zb = G.zb; z.zc = G.zc; z.dzf = G.dzf;
+  z.za = G.za; z.zg = G.zg; z.zc = G.zc; z.dzf = G.dzf;
+  z.dzf64 = G.dzf64; z.zdf = G.zdf;
   z.periodic = G.periodic_z;
   z.singular = G.singular;
   z.skip = nullptr;
@@ -122,6 +125,8 @@ __device__ __forceinline__ df bnb(int kind, bool inner, const double* q, df pc) 
   if (kind == BEND_N) return df{0.f, 0.f};
   return df{-2.f * pc.h, -2.f * pc.l};
 }
+
+__device__ __noinline__ void zsing(const ZArgs<float>& z, float2* cs, float2* ds) { zcolumn_df(z, 0, cs, ds); }
 
 // One residual tile: points [t·chunk, (t+1)·chunk) of grid G, r = (f − μ) − A·Φ in
 // double-float, FP32 r written (unless check), reductions into the grid's words.
@@ -305,10 +310,12 @@ __global__ void __launch_bounds__(256, 4) batch_kernel(BatchArgs A) {
           xform_group<float, float, float, true, 9>(bx_args(G, 1, w, w, 0, nullptr), idx, smem);
           break;
         case BS_Z:
-          zsolve_column<float>(bz_args(G, ws), idx * blockDim.x + threadIdx.x);
-          break;
-        case BS_ZS:
-          zsingular_block<float>(bz_args(G, ws), smem);
+          if (idx < G.ntask[2]) {
+            zsolve_column<float>(bz_args(G, ws), idx * blockDim.x + threadIdx.x);
+          } else if (threadIdx.x < 32) {  // the singular column, by one warp in double-float
+            float2* zs = reinterpret_cast<float2*>(smem);
+            zsing(bz_args(G, ws), zs, zs + G.nz);
+          }
           break;
         case BS_YB:
           xform_group<float, float, float, false, 9>(bx_args(G, 1, w, w, 0, nullptr), idx, smem);
@@ -415,12 +422,12 @@ ps_status build_tables(ps_batch* b) {
   // stage list (same for every grid)
   std::vector<int> stype, sit;
   auto add = [&](int t, int it) { stype.push_back(t); sit.push_back(it); };
-  add(BS_XF64, 0); add(BS_YF, 0); add(BS_Z, 0); add(BS_ZS, 0); add(BS_YB, 0); add(BS_XBST, 0);
+  add(BS_XF64, 0); add(BS_YF, 0); add(BS_Z, 0); add(BS_YB, 0); add(BS_XBST, 0);
   for (int it = 0; it <= b->max_iter; ++it) {
     add(it == b->max_iter ? BS_CHK : BS_RES, it);
     add(BS_FIN, it);
     if (it < b->max_iter) {
-      add(BS_XF, it); add(BS_YF, it); add(BS_Z, it); add(BS_ZS, it); add(BS_YB, it); add(BS_XBACC, it);
+      add(BS_XF, it); add(BS_YF, it); add(BS_Z, it); add(BS_YB, it); add(BS_XBACC, it);
     }
   }
   const int S = (int)stype.size();
@@ -443,8 +450,8 @@ ps_status build_tables(ps_batch* b) {
     B.nalpha = df{(float)(-alpha), (float)(-alpha - (double)(float)(-alpha))};
     B.singular = pn(d.bcx) && pn(d.bcy) && pn(d.bcz) && !B.shift;
     B.periodic_z = d.bcz == PS_BC_PERIODIC;
-    ps_plan_internal_tables(pl, &B.tabx, &B.taby, &B.lamx, &B.lamy, &B.za, &B.zb, &B.zc, &B.dzf, &B.zlo,
-                            &B.zhi, &B.idx2, &B.idy2, &B.wsum_total);
+    ps_plan_internal_tables(pl, &B.tabx, &B.taby, &B.lamx, &B.lamy, &B.za, &B.zg, &B.zc, &B.dzf,
+                            &B.dzf64, &B.zdf, &B.zlo, &B.zhi, &B.idx2, &B.idy2, &B.wsum_total);
     B.mx = d.nx / 2;
     B.my = d.ny / 2;
     const size_t N = (size_t)d.nx * d.ny * d.nz;
@@ -464,7 +471,7 @@ ps_status build_tables(ps_batch* b) {
     B.ntask[3] = (int)((N + B.res_chunk - 1) / B.res_chunk);
     smem = std::max(smem, batch_tile_smem(B.mx, B.lgx));
     smem = std::max(smem, batch_tile_smem(B.my, B.lgy));
-    smem = std::max(smem, 2 * (size_t)d.nz * sizeof(float));
+    if (B.singular) smem = std::max(smem, 2 * (size_t)d.nz * sizeof(float2));
     // workspace slice: partials | w | scr | scr_u
     B.ws_off = ws_off;
     size_t o = a256((N + 2047) / 2048 * 4 * sizeof(float));  // partials for the finest tiling
@@ -480,8 +487,7 @@ ps_status build_tables(ps_batch* b) {
       switch (stype[s]) {
         case BS_XF64: case BS_XF: case BS_XBST: case BS_XBACC: n = B.ntask[0]; break;
         case BS_YF: case BS_YB: n = B.ntask[1]; break;
-        case BS_Z: n = B.ntask[2]; break;
-        case BS_ZS: n = B.singular ? 1 : 0; break;
+        case BS_Z: n = B.ntask[2] + (B.singular ? 1 : 0); break;
         case BS_RES: case BS_CHK: n = B.ntask[3]; break;
         default: n = 1; break;
       }

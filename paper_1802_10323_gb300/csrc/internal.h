@@ -80,24 +80,28 @@ struct ZArgs {
   const T* lamx;            // λ_qx/Δx², nx
   const T* lamy;            // λ_qy/Δy², ny
   const T* za;              // a_k (sub-diagonal; a_0 = wrap coupling when periodic)
-  const T* zb;              // b_k (diagonal incl. Dirichlet ghost terms)
   const T* zc;              // c_k (super-diagonal; c_{n−1} = wrap coupling when periodic)
+  const T* zg;              // excess g_k = −(a_k + b_k + c_k) ≥ 0 of the diagonal without λ (a Dirichlet
+                            // end, the Helmholtz shift), from its terms, not by subtraction
   const T* dzf;             // cell widths (weights of the singular column)
   int periodic;
   int singular;             // column (0,0) is singular: handled by the fix-up kernel
   const int* skip;
-  // FP32 path, non-periodic z: the columns q_x < lowx, q_y < lowy (the worst-conditioned,
-  // see tridiag.cu) are solved in FP64 by extra CTAs of the same launch (0: none).
+  // FP32 path: the columns q_x < lowx, q_y < lowy (the worst-conditioned, see tridiag.cu;
+  // the singular one among them) are solved in double-float by extra CTAs of the same
+  // launch (0: none).
   int lowx, lowy;
-  const double *lamx64, *lamy64, *za64, *zb64, *zc64, *dzf64;
+  const double *lamx64, *lamy64, *dzf64;
+  const float2* zdf;        // per plane (a_k, c_k, g_k) in double-float
+  float ga, ge0, ge1;       // the excess g_k in its terms: every row's (the shift), the first and last row's extra
   double* scr64;            // 2·nz·lowx·lowy doubles
 };
 
-template <class T>
-cudaError_t launch_zsolve(ZArgs<T> a, cudaStream_t st);
-template <class T>
-cudaError_t launch_zsingular(ZArgs<T> a, cudaStream_t st);
-cudaError_t launch_zsolve_ckpt(ZArgs<float> a, cudaStream_t st);  // FP32, non-periodic
+constexpr int ZK = 16;  // planes per checkpoint of the FP32 z sweeps (tridiag.cu)
+__host__ __device__ inline int zckpt_chunks(int rows) { return (rows + ZK - 1) / ZK; }
+cudaError_t launch_zsolve64(ZArgs<double> a, cudaStream_t st);     // FP64, the singular column included
+cudaError_t launch_zsolve_ckpt(ZArgs<float> a, cudaStream_t st);   // FP32
+cudaError_t launch_zsingular(ZArgs<float> a, cudaStream_t st);     // FP32, no rectangle
 
 // Residuals of the refinement (residual.cu): incremental passes on an FP32
 // operand with a double-float base, and the exact pass from the FP64 solution.
@@ -208,8 +212,8 @@ void set_plan_error(ps_plan* plan, const char* msg);
 // The FP32 tables of a plan (used by the batched solve).
 double ps_plan_internal_alpha(const ps_plan* p);  // the plan's Helmholtz shift (0: Poisson)
 void ps_plan_internal_tables(const ps_plan* p, LineTab<float>* tx, LineTab<float>* ty,
-                             const float** lamx, const float** lamy, const float** za, const float** zb,
-                             const float** zc, const float** dzf, const float2** zlo, const float2** zhi,
+                             const float** lamx, const float** lamy, const float** za, const float** zg,
+                             const float** zc, const float** dzf, const double** dzf64, const float2** zdf, const float2** zlo, const float2** zhi,
                              df* idx2, df* idy2, double* wsum_total);
 
 }  // namespace ps

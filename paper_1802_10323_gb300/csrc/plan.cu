@@ -276,16 +276,18 @@ struct ps_plan {
   size_t N;
   AxisTab ax, ay;
   // z tables
-  double *za64, *zb64, *zc64, *dzf64, *idzf64, *idzc64;
-  float *za32, *zb32, *zc32, *dzf32, *idzf32, *idzc32;
+  double *za64, *zg64, *zc64, *dzf64, *idzf64, *idzc64;  // (zg: the excess −(a_k + b_k + c_k))
+  float *za32, *zg32, *zc32, *dzf32, *idzf32, *idzc32;
   float2 *zlo, *zhi;
+  float2* zdf;   // z coefficients (a_k, c_k, g_k) per plane in double-float (rectangle columns)
   float2* zres;  // residual passes m ≥ 1: (a_k, c_k, w_c) per plane, Dirichlet ghost sign folded in
   double asum;   // max over rows of Σ_j |w_j| (those passes' accumulator binade)
   double wsum;  // Σ Δz^f (the per-plane weights of the singular mean, times nx·ny)
   double anorm; // an upper bound of ‖A‖∞ (the drift bound of the incremental residual)
   double alpha = 0.0;  // Helmholtz shift: the plan solves (A − α·I)·p = f
+  double ge0, ge1;     // excess of the z systems' first and last row beyond α (Dirichlet ends)
   df nalpha = {0.f, 0.f};  // −α in double-float (residual pass 0)
-  int lowx, lowy;  // FP32 non-periodic z: rectangle of columns solved in FP64 (tridiag.cu)
+  int lowx, lowy;  // FP32 solves: rectangle of columns solved in double-float (tridiag.cu)
   df idx2, idy2;
   void* dev;    // one allocation for all of the above
   int resid_blocks;     // CTAs of a residual pass (max over the two shapes: partials size)
@@ -342,9 +344,16 @@ WsLayout ws_layout(const ps_plan* p) {
   L.scr_c = off;
   off += align256(p->N * tz);
   L.scr_u = off;
-  if (p->periodic_z) off += align256(p->N * tz);
+  const size_t zlow = align256((size_t)2 * p->nz * p->lowx * p->lowy * sizeof(double));
   L.zlow = off;
-  off += align256((size_t)2 * p->nz * p->lowx * p->lowy * sizeof(double));
+  if (p->periodic_z) {
+    // FP32: the periodic columns' checkpoints fill a small part of this array, and the
+    // rectangle's scratch (at most half of it: lowx·lowy ≤ n_x·n_y/8, n_z ≥ 32) follows them
+    off += align256(p->N * tz);
+    if (zlow) L.zlow = L.scr_u + align256((size_t)zckpt_chunks(p->nz - 1) * p->nx * p->ny * sizeof(float));
+  } else {
+    off += zlow;
+  }
   L.total = off;
   return L;
 }
@@ -384,10 +393,10 @@ ZArgs<T> zargs(const ps_plan* p, T* data, void* ws, const WsLayout& L, const int
   a.nz = p->nz;
   if constexpr (sizeof(T) == 8) {
     a.lamx = p->ax.lam64; a.lamy = p->ay.lam64;
-    a.za = p->za64; a.zb = p->zb64; a.zc = p->zc64; a.dzf = p->dzf64;
+    a.za = p->za64; a.zg = p->zg64; a.zc = p->zc64; a.dzf = p->dzf64;
   } else {
     a.lamx = p->ax.lam32; a.lamy = p->ay.lam32;
-    a.za = p->za32; a.zb = p->zb32; a.zc = p->zc32; a.dzf = p->dzf32;
+    a.za = p->za32; a.zg = p->zg32; a.zc = p->zc32; a.dzf = p->dzf32;
   }
   a.periodic = p->periodic_z;
   a.singular = p->singular;
@@ -397,10 +406,11 @@ ZArgs<T> zargs(const ps_plan* p, T* data, void* ws, const WsLayout& L, const int
     a.lowy = p->lowy;
     a.lamx64 = p->ax.lam64;
     a.lamy64 = p->ay.lam64;
-    a.za64 = p->za64;
-    a.zb64 = p->zb64;
-    a.zc64 = p->zc64;
     a.dzf64 = p->dzf64;
+    a.zdf = p->zdf;
+    a.ga = (float)p->alpha;
+    a.ge0 = (float)p->ge0;
+    a.ge1 = (float)p->ge1;
     a.scr64 = reinterpret_cast<double*>(w + L.zlow);
   }
   return a;
@@ -613,14 +623,14 @@ ps_status solve_plain(ps_plan* pl, const T* f, T* p, void* ws, cudaStream_t st, 
     return cuda_fail(pl, e, "y forward");
   const ZArgs<T> za = yl ? zargs_t<T>(pl, yt, ws, L, nullptr, p) : zargs<T>(pl, p, ws, L, nullptr);
   if ((e = run(pl, K_Z, st, [&] {
-         if constexpr (sizeof(T) == 4)
-           if (!pl->periodic_z) return launch_zsolve_ckpt(za, st);
-         return launch_zsolve<T>(za, st);
+         if constexpr (sizeof(T) == 4) return launch_zsolve_ckpt(za, st);
+         else return launch_zsolve64(za, st);
        })) != cudaSuccess)
     return cuda_fail(pl, e, "z solve");
-  if (pl->singular && !(sizeof(T) == 4 && !pl->periodic_z && pl->lowx > 0) &&
-      (e = run(pl, K_ZS, st, [&] { return launch_zsingular<T>(za, st); })) != cudaSuccess)
-    return cuda_fail(pl, e, "z singular column");
+  if constexpr (sizeof(T) == 4)
+    if (pl->singular && pl->lowx == 0 &&
+        (e = run(pl, K_ZS, st, [&] { return launch_zsingular(za, st); })) != cudaSuccess)
+      return cuda_fail(pl, e, "z singular column");
   if ((e = y_pass<T, false>(pl, K_YB, yl, p, yt, nullptr, st, [&] {
          return line_xform<T, T, T, false>(pl, 1, p, p, nullptr, 0, nullptr, st);
        })) != cudaSuccess)
@@ -691,12 +701,9 @@ ps_status solve_refine(ps_plan* pl, const double* f, double* p, void* ws, cudaSt
     // the planes untransposed)
     const bool ytr = y_long(pl) && !(first && hp);
     const ZArgs<float>& za = ytr ? zwt : zw;
-    if ((r = run(pl, K_Z, st, [&] {
-           return pl->periodic_z ? launch_zsolve<float>(za, st) : launch_zsolve_ckpt(za, st);
-         })) != cudaSuccess)
-      return r;
-    if (pl->singular && (pl->periodic_z || pl->lowx == 0) &&
-        (r = run(pl, K_ZS, st, [&] { return launch_zsingular<float>(za, st); })) != cudaSuccess) return r;
+    if ((r = run(pl, K_Z, st, [&] { return launch_zsolve_ckpt(za, st); })) != cudaSuccess) return r;
+    if (pl->singular && pl->lowx == 0 &&
+        (r = run(pl, K_ZS, st, [&] { return launch_zsingular(za, st); })) != cudaSuccess) return r;
     if ((r = y_pass<float, false>(pl, K_YB, ytr, w, yt, skip, st, [&] {
            return line_xform<float, float, float, false>(pl, 1, w, w, nullptr, 0, skip, st, nullptr, nullptr,
                                                          nullptr, 0, yscr);
@@ -837,15 +844,17 @@ bool take_injected_alloc_failure() {
 double ps_plan_internal_alpha(const ps_plan* p) { return p->alpha; }
 
 void ps_plan_internal_tables(const ps_plan* p, LineTab<float>* tx, LineTab<float>* ty,
-                             const float** lamx, const float** lamy, const float** za, const float** zb,
-                             const float** zc, const float** dzf, const float2** zlo, const float2** zhi,
+                             const float** lamx, const float** lamy, const float** za, const float** zg,
+                             const float** zc, const float** dzf, const double** dzf64, const float2** zdf, const float2** zlo, const float2** zhi,
                              df* idx2, df* idy2, double* wsum_total) {
   *tx = p->ax.gb;
   *ty = p->ay.gb;
   *lamx = p->ax.lam32;
   *lamy = p->ay.lam32;
   *za = p->za32;
-  *zb = p->zb32;
+  *zg = p->zg32;
+  *dzf64 = p->dzf64;
+  *zdf = p->zdf;
   *zc = p->zc32;
   *dzf = p->dzf32;
   *zlo = p->zlo;
@@ -914,6 +923,7 @@ ps_status ps_plan_create_helmholtz(ps_plan** out, int nx, int ny, int nz, double
   for (int k = 0; k < nz; ++k) dzf[k] = faces[k + 1] - faces[k];
   for (int k = 0; k + 1 < nz; ++k) dzc[k] = 0.5 * (faces[k + 2] - faces[k]);
   std::vector<double> lo(nz, 0.0), hi(nz, 0.0);  // residual coefficients
+  double ge0 = 0.0, ge1 = 0.0;                   // −(a_k + b_k + c_k) of the first and last row
   for (int k = 1; k < nz; ++k) za[k] = lo[k] = 1.0 / (dzf[k] * dzc[k - 1]);
   for (int k = 0; k + 1 < nz; ++k) zc[k] = hi[k] = 1.0 / (dzf[k] * dzc[k]);
   for (int k = 0; k < nz; ++k) zb[k] = -(za[k] + zc[k]);
@@ -926,10 +936,12 @@ ps_status ps_plan_create_helmholtz(ps_plan** out, int nx, int ny, int nz, double
   } else {
     if (bcz == PS_BC_DIRICHLET_DIRICHLET || bcz == PS_BC_DIRICHLET_NEUMANN) {
       zb[0] -= 2.0 / (dzf[0] * dzf[0]);
+      ge0 = 2.0 / (dzf[0] * dzf[0]);
       lo[0] = 1.0 / (dzf[0] * dzf[0]);
     }
     if (bcz == PS_BC_DIRICHLET_DIRICHLET || bcz == PS_BC_NEUMANN_DIRICHLET) {
       zb[nz - 1] -= 2.0 / (dzf[nz - 1] * dzf[nz - 1]);
+      ge1 = 2.0 / (dzf[nz - 1] * dzf[nz - 1]);
       hi[nz - 1] = 1.0 / (dzf[nz - 1] * dzf[nz - 1]);
     }
   }
@@ -945,15 +957,26 @@ ps_status ps_plan_create_helmholtz(ps_plan** out, int nx, int ny, int nz, double
     std::fill(hi.begin(), hi.end(), 0.0);
     zb[0] = -1.0;
     lo[0] = 0.5;
+    ge0 = 1.0;
     for (int k = 1; k < nz; ++k) {
       const double h = dzc[k - 1];
       const double dn = 1.0 / (dzf[k - 1] * h), up = 1.0 / (dzf[k] * h);
       za[k] = lo[k] = dn;
       zb[k] = -(dn + up);
-      if (k + 1 < nz) zc[k] = hi[k] = up;
-      else hi[k] = 0.5 * up;
+      if (k + 1 < nz) {
+        zc[k] = hi[k] = up;
+      } else {
+        hi[k] = 0.5 * up;
+        ge1 = up;
+      }
     }
   }
+  // the excess g_k = −(a_k + b_k + c_k) of the z systems' diagonals (with the Helmholtz shift)
+  p->ge0 = ge0;
+  p->ge1 = ge1;
+  std::vector<double> zg(nz, alpha);
+  zg[0] += ge0;
+  zg[nz - 1] += ge1;
   double wsum = 0.0;
   for (int k = 0; k < nz; ++k) {
     split_df(lo[k], &zlo[k]);
@@ -1014,7 +1037,7 @@ ps_status ps_plan_create_helmholtz(ps_plan** out, int nx, int ny, int nz, double
     bytes += gen_table_bytes(bcs[a], n);
   }
   bytes += 6 * align256(nz * sizeof(double)) + 6 * align256(nz * sizeof(float)) +
-           2 * align256(nz * sizeof(float2)) + align256(3 * nz * sizeof(float2));
+           2 * align256(nz * sizeof(float2)) + 2 * align256(3 * nz * sizeof(float2));
   char* dev = nullptr;
   cudaError_t e = take_injected_alloc_failure() ? cudaErrorMemoryAllocation : cudaMalloc(&dev, bytes);
   if (e != cudaSuccess) {
@@ -1026,16 +1049,16 @@ ps_status ps_plan_create_helmholtz(ps_plan** out, int nx, int ny, int nz, double
   p->dev = dev;
   size_t off = 0;
   {
-    // FP32 paths with a non-periodic z: columns whose z system has κ ≈ ‖T_z‖/|λ| > 10^4
-    // are solved in FP64 (tridiag.cu). λ grows with q along each axis, so they lie in
+    // FP32 paths: columns whose z system has κ ≈ ‖T_z‖/|λ| > 10^5 are solved in
+    // double-float (tridiag.cu; a periodic z needs 32 planes for that). λ grows with q along each axis, so they lie in
     // the rectangle q_x < lowx, q_y < lowy; at most 1/8 of the columns. A Helmholtz
     // shift adds α to every |λ| (all terms of the diagonal shift have one sign).
     p->lowx = p->lowy = 0;
-    if (prec != PS_FP64 && bcz != PS_BC_PERIODIC) {
+    if (prec != PS_FP64 && (bcz != PS_BC_PERIODIC || nz >= 32)) {
       double zmax = 0.0;
       for (int k = 0; k < nz; ++k)
         zmax = std::max(zmax, std::fabs(za[k]) + std::fabs(zb[k]) + std::fabs(zc[k]));
-      const double thr = zmax / 1e4;
+      const double thr = zmax / 1e5;
       const std::vector<double> lx = eig_scaled(bcx, nx, dx), ly = eig_scaled(bcy, ny, dy);
       int qx = 0, qy = 0;
       while (qx < nx && std::fabs(lx[qx]) + alpha < thr) ++qx;
@@ -1079,16 +1102,14 @@ ps_status ps_plan_create_helmholtz(ps_plan** out, int nx, int ny, int nz, double
     hput(t.lam32, lam32.data(), n * sizeof(float));
     gen_tables(t, tw64, take, hput);
   }
-  double** d64[6] = {&p->za64, &p->zb64, &p->zc64, &p->dzf64, &p->idzf64, &p->idzc64};
-  float** d32[6] = {&p->za32, &p->zb32, &p->zc32, &p->dzf32, &p->idzf32, &p->idzc32};
+  double** d64[6] = {&p->za64, &p->zg64, &p->zc64, &p->dzf64, &p->idzf64, &p->idzc64};
+  float** d32[6] = {&p->za32, &p->zg32, &p->zc32, &p->dzf32, &p->idzf32, &p->idzc32};
   std::vector<double> idzf(nz), idzc(nz, 0.0);
   for (int k = 0; k < nz; ++k) idzf[k] = 1.0 / dzf[k];
   for (int k = 1; k < nz; ++k) idzc[k] = 1.0 / dzc[k - 1];
   if (bcz == PS_BC_PERIODIC) idzc[0] = 1.0 / (0.5 * (dzf[0] + dzf[nz - 1]));
-  // the z solves' diagonal b_k carries the Helmholtz shift (−α on every row of Eq. 5)
-  std::vector<double> zbs(zb);
-  for (int k = 0; k < nz; ++k) zbs[k] -= alpha;
-  const std::vector<double>* srcs[6] = {&za, &zbs, &zc, &dzf, &idzf, &idzc};
+  // the z solves' excess g_k carries the Helmholtz shift (−α on every diagonal of Eq. 5)
+  const std::vector<double>* srcs[6] = {&za, &zg, &zc, &dzf, &idzf, &idzc};
   for (int i = 0; i < 6; ++i) {
     *d64[i] = reinterpret_cast<double*>(take(nz * sizeof(double)));
     *d32[i] = reinterpret_cast<float*>(take(nz * sizeof(float)));
@@ -1102,6 +1123,15 @@ ps_status ps_plan_create_helmholtz(ps_plan** out, int nx, int ny, int nz, double
   hput(p->zlo, zlo.data(), nz * sizeof(float2));
   hput(p->zhi, zhi.data(), nz * sizeof(float2));
   hput(p->zres, zres.data(), 3 * nz * sizeof(float2));
+  std::vector<float2> zdf(3 * (size_t)nz);
+  for (int k = 0; k < nz; ++k) {
+    split_df(za[k], &zdf[3 * (size_t)k]);
+    split_df(zc[k], &zdf[3 * (size_t)k + 1]);
+    split_df(zg[k], &zdf[3 * (size_t)k + 2]);
+  }
+
+  p->zdf = reinterpret_cast<float2*>(take(3 * nz * sizeof(float2)));
+  hput(p->zdf, zdf.data(), 3 * nz * sizeof(float2));
   e = cudaMemcpy(dev, host.data(), bytes, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     cudaFree(dev);
