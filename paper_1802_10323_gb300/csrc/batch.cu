@@ -184,25 +184,27 @@ __device__ void residual_tile(const BGrid& G, const double* f, const double* p, 
   }
   __syncthreads();
   if (threadIdx.x == 0) {
+    int* red = reinterpret_cast<int*>(c->red);  // (signed keys here, set by reset_red)
     for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
       rmax = fmaxf(rmax, sred[w][0]); rmin = fminf(rmin, sred[w][1]);
       fmx = fmaxf(fmx, sred[w][2]); fmn = fminf(fmn, sred[w][3]);
       wr = df_add(wr, df{sred[w][4], sred[w][5]});
       wf = df_add(wf, df{sred[w][6], sred[w][7]});
     }
-    atomicMax(&c->red[0], f32_key(rmax));
-    atomicMin(&c->red[1], f32_key(rmin));
-    atomicMax(&c->red[2], f32_key(fmx));
-    atomicMin(&c->red[3], f32_key(fmn));
+    atomicMax(&red[0], f32_key(rmax));
+    atomicMin(&red[1], f32_key(rmin));
+    atomicMax(&red[2], f32_key(fmx));
+    atomicMin(&red[3], f32_key(fmn));
     reinterpret_cast<float4*>(partial)[t] = make_float4(wr.h, wr.l, wf.h, wf.l);
   }
 }
 
 __device__ void reset_red(Ctrl* c) {
-  c->red[0] = f32_key(-INFINITY);
-  c->red[1] = f32_key(INFINITY);
-  c->red[2] = f32_key(-INFINITY);
-  c->red[3] = f32_key(INFINITY);
+  int* red = reinterpret_cast<int*>(c->red);
+  red[0] = f32_key(-INFINITY);
+  red[1] = f32_key(INFINITY);
+  red[2] = f32_key(-INFINITY);
+  red[3] = f32_key(INFINITY);
 }
 
 // Convergence test of one grid (one CTA).
@@ -243,8 +245,9 @@ __device__ void finalize_grid(const BGrid& G, Ctrl* c, const float* partial, dou
       mf = c->mf;
     }
   }
-  const double rmax = key_f32(c->red[0]), rmin = key_f32(c->red[1]);
-  const double vmax = key_f32(c->red[2]), vmin = key_f32(c->red[3]);
+  const int* red = reinterpret_cast<const int*>(c->red);
+  const double rmax = key_f32(red[0]), rmin = key_f32(red[1]);
+  const double vmax = key_f32(red[2]), vmin = key_f32(red[3]);
   const double rn = fmax(rmax - mr, mr - rmin), fn = fmax(vmax - mf, mf - vmin);
   const double rel = fn > 0 ? rn / fn : (rn > 0 ? INFINITY : 0.0);
   c->rel = rel; c->rnorm = rn; c->fnorm = fn; c->iterations = it;

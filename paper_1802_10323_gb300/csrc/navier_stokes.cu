@@ -74,6 +74,7 @@ template <class T, bool PX, bool PY, bool PZ>
 __global__ void __launch_bounds__(PTX * PTY, PMINB) ns_predict_kernel(NsArgs<T> a, const T* __restrict__ u3,
                                                                   const T* __restrict__ p, const T* ad_prev,
                                                                   T* __restrict__ ustar, T* ad_out, int zchunk) {
+  pdl_wait();
   using N = NumOf<T>;
   using X = Num<N>;
   struct Slot {
@@ -270,6 +271,7 @@ __global__ void __launch_bounds__(PTX * PTY, PMINB) ns_predict_kernel(NsArgs<T> 
 template <class T>
 __global__ void __launch_bounds__(256) ns_pressure_kernel(size_t N, T scale, T* __restrict__ p,
                                                           T* __restrict__ phi) {
+  pdl_wait();
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < N; g += (size_t)gridDim.x * blockDim.x) {
     const T f = phi[g] * scale;
     phi[g] = f;
@@ -303,27 +305,25 @@ cudaError_t launch_ns_predict(const NsArgs<T>& a, const void* u3, const void* p,
   const int zchunk = (int)((a.nz + nch - 1) / nch);
   const dim3 grid(gx, gy, (a.nz + zchunk - 1) / zchunk);
   auto go = [&](auto k) {
-    k<<<grid, dim3(PTX, PTY), 0, st>>>(a, static_cast<const T*>(u3), static_cast<const T*>(p),
+    return launch_k(k, grid, dim3(PTX, PTY), 0, st, a, static_cast<const T*>(u3), static_cast<const T*>(p),
                                        static_cast<const T*>(ad_prev), static_cast<T*>(ustar),
                                        static_cast<T*>(ad_out), zchunk);
   };
   switch (sel) {
-    case 0: go(ns_predict_kernel<T, false, false, false>); break;
-    case 1: go(ns_predict_kernel<T, true, false, false>); break;
-    case 2: go(ns_predict_kernel<T, false, true, false>); break;
-    case 3: go(ns_predict_kernel<T, true, true, false>); break;
-    case 4: go(ns_predict_kernel<T, false, false, true>); break;
-    case 5: go(ns_predict_kernel<T, true, false, true>); break;
-    case 6: go(ns_predict_kernel<T, false, true, true>); break;
-    default: go(ns_predict_kernel<T, true, true, true>); break;
+    case 0: return go(ns_predict_kernel<T, false, false, false>);
+    case 1: return go(ns_predict_kernel<T, true, false, false>);
+    case 2: return go(ns_predict_kernel<T, false, true, false>);
+    case 3: return go(ns_predict_kernel<T, true, true, false>);
+    case 4: return go(ns_predict_kernel<T, false, false, true>);
+    case 5: return go(ns_predict_kernel<T, true, false, true>);
+    case 6: return go(ns_predict_kernel<T, false, true, true>);
+    default: return go(ns_predict_kernel<T, true, true, true>);
   }
-  return cudaGetLastError();
 }
 
 template <class T>
 cudaError_t launch_ns_pressure(size_t N, double scale, void* p, void* phi, cudaStream_t st) {
-  ns_pressure_kernel<T><<<grid_for(N), 256, 0, st>>>(N, (T)scale, static_cast<T*>(p), static_cast<T*>(phi));
-  return cudaGetLastError();
+  return launch_k(ns_pressure_kernel<T>, grid_for(N), 256, 0, st, N, (T)scale, static_cast<T*>(p), static_cast<T*>(phi));
 }
 
 template cudaError_t launch_ns_predict<float>(const NsArgs<float>&, const void*, const void*, const void*, void*,

@@ -28,6 +28,7 @@ namespace ps {
 
 template <class T>
 __global__ void div_kernel(ProjArgs<T> a, const T* __restrict__ u, T* __restrict__ f) {
+  pdl_wait();
   const size_t N = (size_t)a.nx * a.ny * a.nz;
   const T* __restrict__ ux = u;
   const T* __restrict__ uy = u + N;
@@ -51,6 +52,7 @@ __global__ void div_kernel(ProjArgs<T> a, const T* __restrict__ u, T* __restrict
 template <class T>
 __global__ void grad_correct_kernel(ProjArgs<T> a, const T* __restrict__ us, const T* __restrict__ phi,
                                     T* __restrict__ u) {
+  pdl_wait();
   const size_t N = (size_t)a.nx * a.ny * a.nz;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < N; g += (size_t)gridDim.x * blockDim.x) {
     const int i = (int)(g % a.nx);
@@ -73,6 +75,7 @@ __global__ void grad_correct_kernel(ProjArgs<T> a, const T* __restrict__ us, con
 // h = Gᵀ g (cells)
 template <class T>
 __global__ void grad_adjoint_kernel(ProjArgs<T> a, const T* __restrict__ gu, T* __restrict__ h) {
+  pdl_wait();
   const size_t N = (size_t)a.nx * a.ny * a.nz;
   const T* __restrict__ gx = gu;
   const T* __restrict__ gy = gu + N;
@@ -100,6 +103,7 @@ __global__ void grad_adjoint_kernel(ProjArgs<T> a, const T* __restrict__ gu, T* 
 template <class T>
 __global__ void div_adjoint_correct_kernel(ProjArgs<T> a, const T* __restrict__ gu, const T* __restrict__ s,
                                            T* __restrict__ out) {
+  pdl_wait();
   const size_t N = (size_t)a.nx * a.ny * a.nz;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < N; g += (size_t)gridDim.x * blockDim.x) {
     const int i = (int)(g % a.nx);
@@ -131,12 +135,11 @@ cudaError_t launch_projection(int op, const ProjArgs<T>& a, const void* x0, cons
   const T* a1 = static_cast<const T*>(x1);
   T* o = static_cast<T*>(y);
   switch (op) {
-    case 0: div_kernel<T><<<blocks, threads, 0, st>>>(a, a0, o); break;
-    case 1: grad_correct_kernel<T><<<blocks, threads, 0, st>>>(a, a0, a1, o); break;
-    case 2: grad_adjoint_kernel<T><<<blocks, threads, 0, st>>>(a, a0, o); break;
-    default: div_adjoint_correct_kernel<T><<<blocks, threads, 0, st>>>(a, a0, a1, o); break;
+    case 0: return launch_k(div_kernel<T>, blocks, threads, 0, st, a, a0, o);
+    case 1: return launch_k(grad_correct_kernel<T>, blocks, threads, 0, st, a, a0, a1, o);
+    case 2: return launch_k(grad_adjoint_kernel<T>, blocks, threads, 0, st, a, a0, o);
+    default: return launch_k(div_adjoint_correct_kernel<T>, blocks, threads, 0, st, a, a0, a1, o);
   }
-  return cudaGetLastError();
 }
 
 template cudaError_t launch_projection<float>(int, const ProjArgs<float>&, const void*, const void*, void*, cudaStream_t);

@@ -180,6 +180,14 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N)); }
 
+// The reduction words hold order-preserving unsigned keys whose maximum is taken, the
+// minimum as the maximum of the complement, so that 0 (the state after the memset, and
+// what each finalize leaves for the next pass) is their identity.
+__device__ __forceinline__ unsigned red_max(float f) { return (unsigned)f32_key(f) ^ 0x80000000u; }
+__device__ __forceinline__ unsigned red_min(float f) { return ~red_max(f); }
+__device__ __forceinline__ float red_max_value(unsigned u) { return key_f32((int)(u ^ 0x80000000u)); }
+__device__ __forceinline__ float red_min_value(unsigned u) { return red_max_value(~u); }
+
 // Block reductions of one pass (warp shuffles, then one thread over the warps):
 // max and min of r (and of f when FIRST) into the reduction words, and the
 // per-block double-float weighted sums into the partials.
@@ -213,11 +221,11 @@ __device__ __forceinline__ void resid_reduce(const ResidArgs& a, float rmax, flo
       wrd = add_u(wrd, df{red[w][4], red[w][5]});
       wf = add_u(wf, df{red[w][6], red[w][7]});
     }
-    atomicMax(&a.red[0], f32_key(rmax));
-    atomicMin(&a.red[1], f32_key(rmin));
+    atomicMax(&a.red[0], red_max(rmax));
+    atomicMax(&a.red[1], red_min(rmin));
     if (FIRST) {
-      atomicMax(&a.red[2], f32_key(fmax_));
-      atomicMin(&a.red[3], f32_key(fmin_));
+      atomicMax(&a.red[2], red_max(fmax_));
+      atomicMax(&a.red[3], red_min(fmin_));
     }
     const int bid = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
     reinterpret_cast<float4*>(a.partial)[bid] = make_float4(wrd.h, wrd.l, wf.h, wf.l);
@@ -250,6 +258,7 @@ __global__ void __launch_bounds__(RTHREADS, RPT >= 4 ? 3 : 4) residual_kernel(Re
   using CT = typename std::conditional<SPLIT3, fxp3, fxp>::type;  // a split cell
   constexpr int TY = RWARPS * RPT, W = RTX + 2, CELLS = resid_cells(RPT);
   constexpr int CPT = (CELLS + RTHREADS - 1) / RTHREADS;  // halo cells per thread
+  pdl_wait();
   if (a.skip && *a.skip) return;
   const int nx = a.nx, ny = a.ny, nz = a.nz;
   const size_t sxy = (size_t)nx * ny;
@@ -563,6 +572,7 @@ __global__ void __launch_bounds__(RTHREADS, RPT >= 8 ? 2 : 3) residual_acc_kerne
   constexpr int TY = RWARPS * RPT, ROWS = TY + 2, CELLS = acc_cells(RPT);
   constexpr int NC16 = VEC ? (8 * ROWS + RTHREADS - 1) / RTHREADS : 1;           // 16-byte copies
   constexpr int NC4 = VEC ? 1 : ((RTX + 2) * ROWS + RTHREADS - 1) / RTHREADS;    // 4-byte copies
+  pdl_wait();
   if (a.skip && *a.skip) return;
   const int nx = a.nx, ny = a.ny, nz = a.nz;
   const size_t sxy = (size_t)nx * ny;
@@ -818,18 +828,8 @@ __global__ void __launch_bounds__(RTHREADS, RPT >= 8 ? 2 : 3) residual_acc_kerne
   if (interior) march(std::true_type{});
   else march(std::false_type{});
   cp_wait<0>();
-  resid_reduce<false>(a, rmax, rmin, -INFINITY, INFINITY, wr, df{0.f, 0.f});
-}
-
-// Resets the reduction words of r (and of f in pass 0) before a residual pass.
-__global__ void reset_red_kernel(int* red, const int* skip, int with_f) {
-  if (skip && *skip) return;
-  red[0] = f32_key(-INFINITY);
-  red[1] = f32_key(INFINITY);
-  if (with_f) {
-    red[2] = f32_key(-INFINITY);
-    red[3] = f32_key(INFINITY);
-  }
+  // (the storing repeat of a pass has been reduced by its check)
+  if constexpr (!OUT) resid_reduce<false>(a, rmax, rmin, -INFINITY, INFINITY, wr, df{0.f, 0.f});
 }
 
 namespace {
@@ -868,8 +868,7 @@ cudaError_t launch_kind(const ResidArgs& b, dim3 grid, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  residual_kernel<RPT, KIND><<<grid, dim3(RTX, RWARPS), smem, st>>>(b);
-  return cudaGetLastError();
+  return launch_k(residual_kernel<RPT, KIND>, grid, dim3(RTX, RWARPS), smem, st, b);
 }
 template <int RPT>
 cudaError_t launch_rpt(const ResidArgs& b, int kind, dim3 grid, cudaStream_t st) {
@@ -920,8 +919,7 @@ cudaError_t launch_acc_kind(const ResidArgs& b, dim3 grid, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  residual_acc_kernel<RPT, KIND><<<grid, dim3(RTX, RWARPS), smem, st>>>(b);
-  return cudaGetLastError();
+  return launch_k(residual_acc_kernel<RPT, KIND>, grid, dim3(RTX, RWARPS), smem, st, b);
 }
 template <int RPT, int K>
 cudaError_t launch_acc_out(const ResidArgs& b, bool out, bool vec, dim3 grid, cudaStream_t st) {
@@ -939,7 +937,6 @@ cudaError_t launch_acc_rpt(const ResidArgs& b, int kind, bool out, bool vec, dim
 }
 // Passes m ≥ 1: same grid as the two-level passes (the finalize sums that many partials).
 cudaError_t launch_resid_acc(const ResidArgs& b0, int pass, cudaStream_t st) {
-  reset_red_kernel<<<1, 1, 0, st>>>(b0.red, b0.skip, 0);
   const ResidShape s = resid_shape(b0.nx, b0.ny, b0.nz, RS_ACC);
   ResidArgs b = b0;
   b.zchunk = s.zchunk;
@@ -949,8 +946,7 @@ cudaError_t launch_resid_acc(const ResidArgs& b0, int pass, cudaStream_t st) {
        : s.rpt == 4 ? launch_acc_rpt<4>(b, kind, out, vec, s.grid, st)
                     : launch_acc_rpt<2>(b, kind, out, vec, s.grid, st);
 }
-cudaError_t launch_resid(const ResidArgs& b0, int kind, int reset_f, cudaStream_t st) {
-  reset_red_kernel<<<1, 1, 0, st>>>(b0.red, b0.skip, reset_f);
+cudaError_t launch_resid(const ResidArgs& b0, int kind, cudaStream_t st) {
   if (b0.bcx == BC_FD || b0.bcy == BC_FD) kind |= RK_FACE;
   const ResidShape s = resid_shape(b0.nx, b0.ny, b0.nz, (kind & RK_SPLIT3) ? RS_SPLIT3 : RS_PASS0);
   ResidArgs b = b0;
@@ -974,13 +970,13 @@ cudaError_t launch_residual_inc(const ResidArgs& a, int pass, int split3, cudaSt
   int kind = RK_U32 | RK_FIRST | (split3 ? RK_SPLIT3 : 0) | (a.nalpha.h != 0.f ? RK_SHIFT : 0);
   if (a.singular) kind |= RK_SING;
   if (a.singular && pass == 1) kind |= RK_SUBMU;
-  return launch_resid(a, kind, pass == 0, st);
+  return launch_resid(a, kind, st);
 }
 
 cudaError_t launch_residual_exact(const ResidArgs& a, cudaStream_t st) {
   if (!a.p || !a.r) return cudaErrorInvalidValue;
   return launch_resid(a, RK_SPLIT3 | (a.singular ? (RK_SING | RK_SUBMU) : 0) | (a.nalpha.h != 0.f ? RK_SHIFT : 0),
-                      0, st);
+                      st);
 }
 
 namespace {
@@ -1035,6 +1031,7 @@ __global__ void __launch_bounds__(1024) finalize_kernel(Ctrl* c, const float* pa
                                                         double wsum_total, int singular, double rtol,
                                                         int iteration, int attempt, int last,
                                                         double anorm, const int* skip, ps_info* info) {
+  pdl_wait();
   if ((skip && *skip) || c->converged) return;
   double s1 = 0.0, s2 = 0.0;
   if (singular) sum_partials(partial, nblocks, s1, s2);
@@ -1056,8 +1053,8 @@ __global__ void __launch_bounds__(1024) finalize_kernel(Ctrl* c, const float* pa
     c->bnd += anorm * (ldexp(bits_f64(c->dmax), -39) + ldexp(bits_f64(c->pmax), -52));
   c->dmax_prev = c->dmax;  // the scale of the output repeat of this pass
   c->dmax = 0;             // the next correction's x backward records max|e| here
-  const double rmax = key_f32(c->red[0]), rmin = key_f32(c->red[1]);
-  const double vfmax = key_f32(c->red[2]), vfmin = key_f32(c->red[3]);
+  const double rmax = red_max_value(c->red[0]), rmin = red_min_value(c->red[1]);
+  const double vfmax = red_max_value(c->red[2]), vfmin = red_min_value(c->red[3]);
   const double rn = fmax(rmax - mr, mr - rmin);
   const double fn = fmax(vfmax - mf, mf - vfmin);
   const double rel = fn > 0 ? rn / fn : (rn > 0 ? INFINITY : 0.0);
@@ -1065,8 +1062,12 @@ __global__ void __launch_bounds__(1024) finalize_kernel(Ctrl* c, const float* pa
     const bool redo = ldexp(anorm * bits_f64(c->pmax), -43) > 0.05 * rtol * fn;
     c->skip_redo = redo ? 0 : 1;
     c->nomat0 = 1;
-    if (redo) return;
+    if (redo) {  // the repeated pass reduces f again
+      c->red[0] = c->red[1] = c->red[2] = c->red[3] = 0;
+      return;
+    }
   }
+  c->red[0] = c->red[1] = 0;  // for the next pass (max and min of f stay)
   c->rnorm = rn;
   c->fnorm = fn;
   c->rel = rel;
@@ -1090,13 +1091,14 @@ __global__ void __launch_bounds__(1024) finalize_kernel(Ctrl* c, const float* pa
 __global__ void __launch_bounds__(1024) finalize_exact_kernel(Ctrl* c, const float* partial, int nblocks,
                                                               double wsum_total, int singular,
                                                               double rtol, ps_info* info) {
+  pdl_wait();
   if (c->vskip) return;
   double s1 = 0.0, s2 = 0.0;
   if (singular) sum_partials(partial, nblocks, s1, s2);
   if (threadIdx.x != 0) return;
   const double mr = singular ? s1 / wsum_total : 0.0, mf = singular ? c->mf : 0.0;
-  const double rmax = key_f32(c->red[0]), rmin = key_f32(c->red[1]);
-  const double vfmax = key_f32(c->red[2]), vfmin = key_f32(c->red[3]);
+  const double rmax = red_max_value(c->red[0]), rmin = red_min_value(c->red[1]);
+  const double vfmax = red_max_value(c->red[2]), vfmin = red_min_value(c->red[3]);
   const double rn = fmax(rmax - mr, mr - rmin);
   const double fn = fmax(vfmax - mf, mf - vfmin);
   const double rel = fn > 0 ? rn / fn : (rn > 0 ? INFINITY : 0.0);
@@ -1115,29 +1117,28 @@ __global__ void __launch_bounds__(1024) finalize_exact_kernel(Ctrl* c, const flo
 cudaError_t launch_finalize(Ctrl* ctrl, const float* partial, int nblocks, double wsum_total,
                             int singular, double rtol, int iteration, int attempt, int last,
                             double anorm, const int* skip, ps_info* info, cudaStream_t st) {
-  finalize_kernel<<<1, 1024, 0, st>>>(ctrl, partial, nblocks, wsum_total, singular, rtol, iteration,
-                                      attempt, last, anorm, skip, info);
-  return cudaGetLastError();
+  return launch_k(finalize_kernel, 1, 1024, 0, st, ctrl, partial, nblocks, wsum_total, singular, rtol, iteration,
+                  attempt, last, anorm, skip, info);
 }
 
 cudaError_t launch_finalize_exact(Ctrl* ctrl, const float* partial, int nblocks, double wsum_total,
                                   int singular, double rtol, ps_info* info, cudaStream_t st) {
-  finalize_exact_kernel<<<1, 1024, 0, st>>>(ctrl, partial, nblocks, wsum_total, singular, rtol, info);
-  return cudaGetLastError();
+  return launch_k(finalize_exact_kernel, 1, 1024, 0, st, ctrl, partial, nblocks, wsum_total, singular, rtol, info);
 }
 
 __global__ void widen_kernel(const float* __restrict__ u, double* __restrict__ p, size_t n, const int* skip) {
+  pdl_wait();
   if (*skip) return;
   for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < n; g += (size_t)gridDim.x * blockDim.x)
     p[g] = widen_f32(u[g]);
 }
 
 cudaError_t launch_widen(const float* u, double* p, size_t n, const int* skip, cudaStream_t st) {
-  widen_kernel<<<152 * 8, 256, 0, st>>>(u, p, n, skip);
-  return cudaGetLastError();
+  return launch_k(widen_kernel, 152 * 8, 256, 0, st, u, p, n, skip);
 }
 
 __global__ void info_plain_kernel(ps_info* info) {
+  pdl_wait();
   info->status = PS_OK;
   info->iterations = 0;
   info->rel_residual = -1.0;
@@ -1146,8 +1147,7 @@ __global__ void info_plain_kernel(ps_info* info) {
 }
 
 cudaError_t launch_info_plain(ps_info* info, cudaStream_t st) {
-  info_plain_kernel<<<1, 1, 0, st>>>(info);
-  return cudaGetLastError();
+  return launch_k(info_plain_kernel, 1, 1, 0, st, info);
 }
 
 }  // namespace ps

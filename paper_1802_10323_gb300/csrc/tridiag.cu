@@ -88,12 +88,13 @@ __device__ __forceinline__ void st_pol(float* p, float v, uint64_t pol) {
 // ONE: columns of at most ZK rows, read once and without a checkpoint.
 template <bool TAB, bool PER, bool ONE>
 __device__ __forceinline__ void zsolve_ckpt(const ZArgs<float>& a, int nlowb) {
-  if (a.skip && *a.skip) return;
   int bulk = blockIdx.x;
   if (nlowb > 0) {
     const int lo = (int)((long long)blockIdx.x * nlowb / gridDim.x);
     const int hi = (int)((long long)(blockIdx.x + 1) * nlowb / gridDim.x);
     if (hi > lo) {
+      pdl_wait();
+      if (a.skip && *a.skip) return;
       zlow_column(a, lo * (ZB / 32) + (threadIdx.x >> 5));
       return;
     }
@@ -110,8 +111,10 @@ __device__ __forceinline__ void zsolve_ckpt(const ZArgs<float>& a, int nlowb) {
   };
   if constexpr (TAB) {
     for (int k = threadIdx.x; k < nz; k += ZB) ztab[k] = coef_of(k);
-    __syncthreads();
   }
+  pdl_wait();
+  if (a.skip && *a.skip) return;
+  if constexpr (TAB) __syncthreads();
   const int ncol = a.nx * a.ny;
   // checkpoints: [nchunk][ncol] of (G, V), and of F when periodic (in the second scratch)
   float2* __restrict__ ck = reinterpret_cast<float2*>(a.scr_c);
@@ -269,8 +272,7 @@ namespace {
 template <bool TAB, bool PER, bool ONE>
 cudaError_t launch_ckpt(const ZArgs<float>& a, int grid, int nlowb, size_t smem, cudaStream_t st) {
   auto k = PER ? zsolve_ckpt_per_kernel<TAB, ONE> : zsolve_ckpt_kernel<TAB, ONE>;
-  k<<<grid, ZB, smem, st>>>(a, nlowb);
-  return cudaGetLastError();
+  return launch_k(k, grid, ZB, smem, st, a, nlowb);
 }
 }  // namespace
 
@@ -298,6 +300,7 @@ cudaError_t launch_zsolve_ckpt(ZArgs<float> a, cudaStream_t st) {
 // 3.4 warps per sub-partition taking the time of four).
 constexpr int ZPART_COLS = 8192;
 __global__ void __launch_bounds__(128) zsolve64_kernel(ZArgs<double> a) {
+  pdl_wait();
   int b = blockIdx.x;
   if (a.singular) {
     if (b == 0) {
@@ -310,6 +313,7 @@ __global__ void __launch_bounds__(128) zsolve64_kernel(ZArgs<double> a) {
 }
 
 __global__ void __launch_bounds__(128) zpart64_kernel(ZArgs<double> a) {
+  pdl_wait();
   const int col = blockIdx.x * 4 + (threadIdx.x >> 5);
   if (col < a.nx * a.ny) zpart64(a, col, a.singular && col == 0);
 }
@@ -317,6 +321,7 @@ __global__ void __launch_bounds__(128) zpart64_kernel(ZArgs<double> a) {
 // FP32 plans without a rectangle (tiny planes, or a periodic z of fewer than 32 planes): the
 // singular column in double-float by one warp
 __global__ void __launch_bounds__(32) zsingular_kernel(ZArgs<float> a) {
+  pdl_wait();
   if (a.skip && *a.skip) return;
   extern __shared__ __align__(16) float2 zsm[];
   zcolumn_df(a, 0, zsm, zsm + a.nz);
@@ -325,10 +330,8 @@ __global__ void __launch_bounds__(32) zsingular_kernel(ZArgs<float> a) {
 cudaError_t launch_zsolve64(ZArgs<double> a, cudaStream_t st) {
   const int ncol = a.nx * a.ny;
   if (ncol <= ZPART_COLS && (!a.periodic || a.nz >= 32))
-    zpart64_kernel<<<(ncol + 3) / 4, 128, 0, st>>>(a);
-  else
-    zsolve64_kernel<<<(ncol + 127) / 128 + (a.singular ? 1 : 0), 128, 0, st>>>(a);
-  return cudaGetLastError();
+    return launch_k(zpart64_kernel, (ncol + 3) / 4, 128, 0, st, a);
+  return launch_k(zsolve64_kernel, (ncol + 127) / 128 + (a.singular ? 1 : 0), 128, 0, st, a);
 }
 
 cudaError_t launch_zsingular(ZArgs<float> a, cudaStream_t st) {
@@ -336,8 +339,7 @@ cudaError_t launch_zsingular(ZArgs<float> a, cudaStream_t st) {
   auto k = zsingular_kernel;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k<<<1, 32, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_k(k, 1, 32, smem, st, a);
 }
 
 }  // namespace ps

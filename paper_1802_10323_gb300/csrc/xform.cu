@@ -5,6 +5,7 @@ namespace ps {
 
 template <class T, class TI, class TO, bool FWD>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2) xform_kernel(XformArgs<T> a) {
+  pdl_wait();
   if (a.skip && *a.skip) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   xform_group<T, TI, TO, FWD>(a, blockIdx.x, smem_raw);
@@ -43,8 +44,7 @@ cudaError_t launch_xform(XformArgs<T> a, cudaStream_t st) {
   auto k = xform_kernel<T, TI, TO, FWD>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k<<<(unsigned)tiles(lg), threads, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_k(k, (unsigned)tiles(lg), threads, smem, st, a);
 }
 
 template cudaError_t launch_xform<double, double, double, true>(XformArgs<double>, cudaStream_t);

@@ -24,7 +24,6 @@ namespace col {
 template <class T, int M, bool FWD, int CW>
 __global__ void __launch_bounds__(CShape<M, CW>::NT, sizeof(T) == 4 ? 1024 / CShape<M, CW>::NT : 1)
     xform_col_kernel(FastArgs<T> a) {
-  if (a.skip && *a.skip) return;
   static_assert(CShape<M, CW>::radix(0) == CShape<M, CW>::E, "the first stage takes all of a thread's points");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx<T>* stw = reinterpret_cast<cplx<T>*>(smem_raw);  // ω_M^t, t < M
@@ -32,6 +31,8 @@ __global__ void __launch_bounds__(CShape<M, CW>::NT, sizeof(T) == 4 ? 1024 / CSh
   cplx<T>* xtw = ptw + (M + 1);                         // NN/DD: e^{−iπq/2n}, q < n; ND: pre, post
   cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw + fast_table_bytes<T, M>(a.bc));  // [M][CW]
   load_line_tables<T, M>(a.tw, a.bc, stw);
+  pdl_wait();
+  if (a.skip && *a.skip) return;
   const int ntiles = a.nz * (a.nx / CW);
   const int tpz = a.nx / CW;
   for (int g = blockIdx.x; g < ntiles; g += gridDim.x) {
@@ -76,8 +77,7 @@ cudaError_t launch_col_cw(FastArgs<T> a, cudaStream_t st) {
   const int ntiles = a.nz * (a.nx / CW);
   const int grid = ntiles < sms * bps ? ntiles : sms * bps;
   (void)cudaGetLastError();  // a stale error from elsewhere must not be blamed here
-  k<<<grid, S::NT, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_k(k, grid, S::NT, smem, st, a);
 }
 }  // namespace
 

@@ -31,6 +31,7 @@ using fast::cpad;
 
 template <class T, class TI, class TO, int M, bool FWD>
 __global__ void __launch_bounds__(512, sizeof(T) == 4 ? 2 : 1) xform_fast_kernel(FastArgs<T> a) {
+  pdl_wait();
   if (a.skip && *a.skip) return;
   constexpr int N = 2 * M;
   constexpr int E = Shape<M>::E, TPL = Shape<M>::TPL;
@@ -432,8 +433,7 @@ cudaError_t launch_xform_fast(FastArgs<T> a, cudaStream_t st) {
   const int ngroups = (a.axis == 0) ? (a.nlines + a.lpc - 1) / a.lpc : a.nz * (a.nx / a.lpc);
   const int grid = min(ngroups, sms * bps);
   cudaError_t pre = cudaGetLastError();  // a stale error from elsewhere must not be blamed here
-  k<<<grid, threads, smem, st>>>(a);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_k(k, grid, threads, smem, st, a);
   if (e != cudaSuccess || pre != cudaSuccess) {
     cudaFuncAttributes fa{};
     cudaFuncGetAttributes(&fa, k);

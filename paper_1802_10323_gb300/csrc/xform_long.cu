@@ -158,13 +158,14 @@ __global__ void __launch_bounds__(LShape<M>::NT, (sizeof(T) == 8 ? 256 : PS_LONG
     xform_long_kernel(FastArgs<T> a) {
   using S = LShape<M>;
   constexpr int N = 2 * M, NT = S::NT, E = S::E, RL = S::radix(S::NST - 1);
-  if (a.skip && *a.skip) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   LTab<T, M> tb;
   tb.carve(reinterpret_cast<cplx<T>*>(smem_raw), a.tw);
   cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw) + LTab<T, M>::ENTRIES;  // [lpad(M) + 1]
   const int b = threadIdx.x;
   tb.fill(b, NT);
+  pdl_wait();
+  if (a.skip && *a.skip) return;
   __syncthreads();  // the tables are complete before the first line's gather reads them
   const cplx<T> tw1 = a.tw[1];  // e^{−2πi/(8n)}: the ND post-twiddle is tw(4k)·tw1
   const int bc = a.bc;
@@ -423,6 +424,7 @@ template <class T>
 __global__ void __launch_bounds__(256) transpose_kernel(const T* __restrict__ src, T* __restrict__ dst, int rows,
                                                         int cols, const int* skip) {
   using T2 = typename std::conditional<sizeof(T) == 4, float2, double2>::type;
+  pdl_wait();
   if (skip && *skip) return;
   extern __shared__ __align__(16) unsigned char tsm[];
   T(*tile)[65] = reinterpret_cast<T(*)[65]>(tsm);  // [64][65]
@@ -476,8 +478,7 @@ cudaError_t launch_long_mode(FastArgs<T> a, cudaStream_t st) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int grid = a.nlines < sms * bps ? a.nlines : sms * bps;
   if (grid <= 0) return cudaSuccess;
-  k<<<grid, S::NT, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_k(k, grid, S::NT, smem, st, a);
 }
 }  // namespace
 
@@ -499,8 +500,7 @@ cudaError_t launch_plane_transpose(const T* src, T* dst, int rows, int cols, int
   if ((rows | cols) & 1) return cudaErrorInvalidValue;  // pairs of consecutive values
   const dim3 grid((cols + 63) / 64, (rows + 63) / 64, nz);
   const size_t smem = 64 * 65 * sizeof(T);  // ≤ 33 KB: no opt-in needed
-  lng::transpose_kernel<T><<<grid, dim3(32, 8), smem, st>>>(src, dst, rows, cols, skip);
-  return cudaGetLastError();
+  return launch_k(lng::transpose_kernel<T>, grid, dim3(32, 8), smem, st, src, dst, rows, cols, skip);
 }
 
 #define PS_LONG_INST(M)                                                                                   \

@@ -26,7 +26,6 @@ namespace row {
 template <class T, class TI, class TO, int M, bool FWD, int OM>
 __global__ void __launch_bounds__(32 * WARPS, sizeof(T) == 4 ? (M >= 512 ? 3 : 4) : 2)
     xform_row_kernel(FastArgs<T> a) {
-  if (a.skip && *a.skip) return;
   constexpr int LPW = 32 / Shape<M>::TPL;
   constexpr int LB = M + M / 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -35,6 +34,8 @@ __global__ void __launch_bounds__(32 * WARPS, sizeof(T) == 4 ? (M >= 512 ? 3 : 4
   cplx<T>* xtw = ptw + (M + 1);
   cplx<T>* bufs = reinterpret_cast<cplx<T>*>(smem_raw + fast_table_bytes<T, M>(a.bc));
   load_line_tables<T, M>(a.tw, a.bc, stw);
+  pdl_wait();
+  if (a.skip && *a.skip) return;
   __syncthreads();  // the only block-wide barrier: tables ready
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // max |transform output| of FP64 outputs, tracked on the values before widening
@@ -84,8 +85,7 @@ cudaError_t launch_row_mode(FastArgs<T> a, cudaStream_t st) {
   const int ctas = (a.nlines + per_cta - 1) / per_cta;
   const int grid = ctas < sms * bps ? ctas : sms * bps;
   (void)cudaGetLastError();  // a stale error from elsewhere must not be blamed here
-  k<<<grid, 32 * row::WARPS, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_k(k, grid, 32 * row::WARPS, smem, st, a);
 }
 }  // namespace
 
