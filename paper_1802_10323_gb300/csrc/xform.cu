@@ -1,5 +1,5 @@
 // xform.cu — launchers of the generic line transforms (device code in xform_dev.cuh).
-#include "xform_dev.cuh"
+#include "xform_mid.cuh"
 
 namespace ps {
 
@@ -20,12 +20,53 @@ size_t tile_smem(int m, int lgL, size_t csize) {
 }
 }  // namespace
 
+namespace {
+// Half lengths with a compile-time kernel (xform_mid_*.cu).
+template <class TI, class TO, int AXIS, bool FWD, int M>
+cudaError_t mid_case(const XformArgs<float>& a, cudaStream_t st, bool* done) {
+  const int L = mid::DimCt<M>::L;
+  const long long tiles = AXIS == 0 ? (a.nlines + L - 1) / L : (long long)a.nz * ((a.nx + L - 1) / L);
+  if (tiles < 152) return cudaSuccess;
+  *done = true;
+  return launch_xform_mid<TI, TO, M, AXIS, FWD>(a, (int)tiles, st);
+}
+// FP32 lines: the kernel with the length at compile time, where the grid gives every SM a
+// tile of it (fewer tiles: the run-time kernel, whose tiles shrink with the grid).
+// 384×288×201 in µs, run-time → compile-time length: x 97 → 73 forward, 99 → 75 backward (into
+// FP32 Φ_0), 160 → 136 (into p), y 113 → 54 and 105 → 56; 192×96×65 solve 45 → 32.
+template <class TI, class TO, int AXIS, bool FWD>
+cudaError_t launch_mid_if(const XformArgs<float>& a, cudaStream_t st, bool* done) {
+  *done = false;
+  if (a.bc == BC_FD) return cudaSuccess;
+  switch (a.m) {
+#define PS_MID_CASE(M) \
+  case M: return mid_case<TI, TO, AXIS, FWD, M>(a, st, done);
+    PS_MID_CASE(16) PS_MID_CASE(18) PS_MID_CASE(24) PS_MID_CASE(27) PS_MID_CASE(32) PS_MID_CASE(36) PS_MID_CASE(48)
+    PS_MID_CASE(54) PS_MID_CASE(72) PS_MID_CASE(81) PS_MID_CASE(96) PS_MID_CASE(108) PS_MID_CASE(144)
+    PS_MID_CASE(162) PS_MID_CASE(192) PS_MID_CASE(216) PS_MID_CASE(243) PS_MID_CASE(288) PS_MID_CASE(324)
+    PS_MID_CASE(384) PS_MID_CASE(432) PS_MID_CASE(486)
+#undef PS_MID_CASE
+    default: return cudaSuccess;
+  }
+}
+}  // namespace
+
 // Lines per tile: 16 (a 64-byte row segment of FP32 y lines, full half-warps) while four
 // CTAs fit an SM (56 KB each); fewer on long lines, down to four (FP32: one 16-byte part of
 // a sector) as long as a CTA's shared memory holds them; and fewer, down to four, while the
 // tiles would leave SMs without work: on a 32^3 grid 16 lines make 64 tiles, four make 256.
 template <class T, class TI, class TO, bool FWD>
 cudaError_t launch_xform(XformArgs<T> a, cudaStream_t st) {
+  if constexpr (sizeof(T) == 4) {
+    bool done = false;
+    cudaError_t e = cudaSuccess;
+    if (a.axis == 0) {
+      e = launch_mid_if<TI, TO, 0, FWD>(a, st, &done);
+    } else if constexpr (sizeof(TI) == 4 && sizeof(TO) == 4) {
+      if (!a.accumulate) e = launch_mid_if<TI, TO, 1, FWD>(a, st, &done);
+    }
+    if (e != cudaSuccess || done) return e;
+  }
   constexpr size_t C = sizeof(cplx<T>);
   constexpr size_t kBest = 56 * 1024, kMost = 220 * 1024;
   auto tiles = [&](int lg) -> long long {

@@ -169,32 +169,57 @@ __device__ __forceinline__ void st_pair(V* p, bool al, V a, V b) {
   }
 }
 
+// The sizes of a tile, at run time (this kernel) or compile time (xform_mid.cuh).
+struct DimRt {
+  int n_, m_, lg_, ls_;
+  unsigned mg_m, mg_h;
+  __device__ __forceinline__ int n() const { return n_; }
+  __device__ __forceinline__ int m() const { return m_; }
+  __device__ __forceinline__ int lg() const { return lg_; }   // log2 of the lines
+  __device__ __forceinline__ int ls() const { return ls_; }   // row pitch of the slots
+  __device__ __forceinline__ int div_m(int i) const { return div_mg(i, mg_m); }
+  __device__ __forceinline__ int div_h(int i) const { return div_mg(i, mg_h); }  // by n/2
+};
+
+// The three kinds of boundary pair, as far as the slots go. by_kind(bc, f) calls f with the
+// kind as a constant, so that loops over values are compiled per kind.
+enum { KIND_P = 0, KIND_CT = 1 /* NN, DD */, KIND_IV = 2 /* ND, DN */ };
+template <class F>
+__device__ __forceinline__ void by_kind(int bc, F&& f) {
+  if (bc == BC_P) f(std::integral_constant<int, KIND_P>{});
+  else if (bc_iv(bc)) f(std::integral_constant<int, KIND_IV>{});
+  else f(std::integral_constant<int, KIND_CT>{});
+}
+
 // Where the line elements sit in the slots. Physical side (the field's values): the
-// elements (e0, e1) of slot p's two parts, and the signs of the DST ordering.
+// elements (e0, e1) of slot p's two parts; spectral side: the coefficients (q0, q1) of slot
+// k's; and the inverse maps for the pair (e, e + 1), e even: slot s and part c of each.
+template <class D, int KIND>
 struct SlotMap {
-  int n, m, bc;
-  __device__ __forceinline__ int mk(int j) const { return j < m ? 2 * j : 2 * n - 1 - 2 * j; }  // Makhoul (n = 2m)
+  D d;
+  int bc;
+  __device__ __forceinline__ int mk(int j) const {  // Makhoul (n = 2m)
+    return j < d.m() ? 2 * j : 2 * d.n() - 1 - 2 * j;
+  }
   __device__ __forceinline__ void phys(int p, int& e0, int& e1) const {
-    if (bc == BC_P) {
+    if constexpr (KIND == KIND_P) {
       e0 = 2 * p;
       e1 = 2 * p + 1;
-    } else if (bc == BC_ND) {
-      e0 = 2 * p;
-      e1 = n - 1 - 2 * p;
-    } else if (bc == BC_DN) {  // the reversed line: the two parts trade places
-      e0 = n - 1 - 2 * p;
-      e1 = 2 * p;
+    } else if constexpr (KIND == KIND_IV) {  // DN, the reversed line: the two parts trade places
+      const int lo = 2 * p, hi = d.n() - 1 - 2 * p;
+      e0 = bc == BC_DN ? hi : lo;
+      e1 = bc == BC_DN ? lo : hi;
     } else {
       e0 = mk(2 * p);
       e1 = mk(2 * p + 1);
     }
   }
-  // spectral side: the coefficients (q0, q1) of slot k's two parts
   __device__ __forceinline__ void spec(int k, int& q0, int& q1) const {
-    if (bc == BC_P) {
+    const int n = d.n(), m = d.m();
+    if constexpr (KIND == KIND_P) {
       q0 = k == 0 ? 0 : 2 * k - 1;
       q1 = k == 0 ? n - 1 : 2 * k;
-    } else if (bc_iv(bc)) {
+    } else if constexpr (KIND == KIND_IV) {
       q0 = 2 * k;
       q1 = n - 1 - 2 * k;
     } else {
@@ -206,14 +231,13 @@ struct SlotMap {
       }
     }
   }
-  // the inverse maps for the pair (e, e + 1), e even: slot s and part c of each
   __device__ __forceinline__ void phys_of(int e, int& s0, int& c0, int& s1, int& c1) const {
-    const int h = e >> 1;
-    if (bc == BC_P) {
+    const int h = e >> 1, n = d.n(), m = d.m();
+    if constexpr (KIND == KIND_P) {
       s0 = s1 = h;
       c0 = 0;
       c1 = 1;
-    } else if (bc_iv(bc)) {
+    } else if constexpr (KIND == KIND_IV) {
       s0 = h;
       s1 = m - 1 - h;
       c0 = bc == BC_DN;
@@ -226,25 +250,204 @@ struct SlotMap {
       c1 = j1 & 1;
     }
   }
-  __device__ __forceinline__ void spec_one(int e, int& s, int& c) const {
-    if (bc == BC_P) {
-      const int k = (e + 1) >> 1;
-      s = k == m ? 0 : k;
-      c = e == 0 ? 0 : (k == m ? 1 : !(e & 1));
-    } else if (bc_iv(bc)) {
-      c = e & 1;
-      s = c ? (n - 1 - e) >> 1 : e >> 1;
+  __device__ __forceinline__ void spec_of(int e, int& s0, int& c0, int& s1, int& c1) const {
+    const int n = d.n(), m = d.m(), h = e >> 1;
+    if constexpr (KIND == KIND_P) {  // X_2h is part 1 of slot h, X_{2h+1} part 0 of slot h + 1; X_0, X_{n−1} in slot 0
+      s0 = h;
+      c0 = h > 0;
+      s1 = h + 1 == m ? 0 : h + 1;
+      c1 = h + 1 == m;
+    } else if constexpr (KIND == KIND_IV) {
+      s0 = h;
+      c0 = 0;
+      s1 = m - 1 - h;
+      c1 = 1;
     } else {
-      const int q = bc == BC_DD ? n - 1 - e : e;
-      c = q >= m;
-      s = q == m ? 0 : (c ? n - q : q);
+      auto one = [&](int q, int& s, int& c) {
+        c = q >= m;
+        s = q == m ? 0 : (c ? n - q : q);
+      };
+      one(bc == BC_DD ? n - 1 - e : e, s0, c0);
+      one(bc == BC_DD ? n - 2 - e : e + 1, s1, c1);
     }
   }
-  __device__ __forceinline__ void spec_of(int e, int& s0, int& c0, int& s1, int& c1) const {
-    spec_one(e, s0, c0);
-    spec_one(e + 1, s1, c1);
-  }
 };
+
+// ---- the steps shared with the compile-time kernels (xform_mid.cuh) ----------------------
+
+// x lines into the slots (FWD: field values, else coefficients): pairs of consecutive
+// values, the lanes along the line.
+template <class D, class T, class TI, bool FWD, class Scale>
+__device__ __forceinline__ void x_load(const D& d, int bc, const TI* in, int live, T* rA, bool scaled, Scale&& scale_of) {
+  const int m = d.m(), ls = d.ls();
+  const bool al = !((uintptr_t)in & (2 * sizeof(TI) - 1));
+  const T sg = (FWD && bc == BC_DD) ? (T)-1 : (T)1;  // DST ordering: the odd elements change sign
+  by_kind(bc, [&](auto kind) {
+    constexpr int KIND = decltype(kind)::value;
+    const SlotMap<D, KIND> map{d, bc};
+#pragma unroll 4
+    for (int idx = threadIdx.x; idx < live * m; idx += blockDim.x) {
+      const int l = d.div_m(idx), e = 2 * (idx - l * m);
+      TI u0, u1;
+      ld_pair(in + 2 * idx, al, u0, u1);
+      T v0 = ld_cvt<T, TI>::f(u0), v1 = ld_cvt<T, TI>::f(u1);
+      if (scaled) {
+        const T sc = scale_of(l);
+        v0 *= sc;
+        v1 *= sc;
+      }
+      if constexpr (FWD && KIND == KIND_P) {  // the pair is one slot
+        reinterpret_cast<cplx<T>*>(rA)[(e >> 1) * ls + l] = {v0, v1};
+      } else {
+        int s0, c0, s1, c1;
+        if (FWD) map.phys_of(e, s0, c0, s1, c1);
+        else map.spec_of(e, s0, c0, s1, c1);
+        rA[2 * (s0 * ls + l) + c0] = v0;
+        rA[2 * (s1 * ls + l) + c1] = (FWD && KIND == KIND_CT) ? sg * v1 : v1;
+      }
+    }
+  });
+}
+
+// Backward P, NN, DD: the pairs (k, m−k), the parts traded for the inverse FFT:
+// Z_k = (V_k + conj V_{m−k})/2m + pb_k·(V_k − conj V_{m−k}), pb_k = i·e^{+2πik/n}/2m; NN, DD:
+// V_q = xb_q·(X_q − i X_{n−q}), xb_q = ½e^{+iπq/2n}. get(k, l): the two values of slot k.
+template <class D, class T, class Get>
+__device__ __forceinline__ void pairs_bwd(const D& d, int bc, cplx<T>* buf, const cplx<T>* t0, const cplx<T>* t1, T s,
+                                          Get&& get) {
+  const int m = d.m(), lg = d.lg(), ls = d.ls(), np = m / 2 + 1;
+#pragma unroll 1
+  for (int idx = threadIdx.x; idx < (np << lg); idx += blockDim.x) {
+    const int l = idx & ((1 << lg) - 1), k = idx >> lg;
+    const cplx<T> x = get(k, l), y = get(k == 0 ? 0 : m - k, l);
+    cplx<T> V, W;
+    if (bc == BC_P) {
+      V = k == 0 ? cplx<T>{x.x, (T)0} : cplx<T>{x.x, -x.y};
+      W = k == 0 ? cplx<T>{x.y, (T)0} : cplx<T>{y.x, -y.y};
+    } else {
+      V = cmul(ldg_c(t1 + k), k == 0 ? cplx<T>{x.x, (T)0} : cplx<T>{x.x, -x.y});
+      W = cmul(ldg_c(t1 + m - k), k == 0 ? cplx<T>{x.y, -x.y} : cplx<T>{y.x, -y.y});
+    }
+    const cplx<T> Sm = cadd(V, conj_(W)), Dm = cmul(ldg_c(t0 + k), csub(V, conj_(W)));
+    buf[k * ls + l] = {s * Sm.y + Dm.y, s * Sm.x + Dm.x};
+    if (k != 0 && 2 * k != m) buf[(m - k) * ls + l] = {Dm.y - s * Sm.y, s * Sm.x - Dm.x};
+  }
+}
+
+// Forward P, NN, DD: the real DFT of the packed sequence,
+// V_k = (Z_k + conj Z_{m−k})/2 + pf_k·(Z_k − conj Z_{m−k}), pf_k = −(i/2)e^{−2πik/n}; NN, DD:
+// X_q = Re(xf_q V_q), X_{n−q} = −Im, xf_q = 2e^{−iπq/2n}. put(k, l, v0, v1): slot k's outputs.
+template <class D, class T, class Put>
+__device__ __forceinline__ void pairs_fwd(const D& d, int bc, const cplx<T>* buf, const cplx<T>* t0,
+                                          const cplx<T>* t1, Put&& put) {
+  const int m = d.m(), lg = d.lg(), ls = d.ls(), np = m / 2 + 1;
+#pragma unroll 1
+  for (int idx = threadIdx.x; idx < (np << lg); idx += blockDim.x) {
+    const int l = idx & ((1 << lg) - 1), k = idx >> lg;
+    const cplx<T> Zk = buf[k * ls + l], Zm = buf[(k == 0 ? 0 : m - k) * ls + l];
+    const cplx<T> Sm = cadd(Zk, conj_(Zm)), Dm = cmul(ldg_c(t0 + k), csub(Zk, conj_(Zm)));
+    const cplx<T> V = {(T)0.5 * Sm.x + Dm.x, (T)0.5 * Sm.y + Dm.y};
+    const cplx<T> W = {(T)0.5 * Sm.x - Dm.x, Dm.y - (T)0.5 * Sm.y};  // V_{m−k}
+    if (bc == BC_P) {
+      if (k == 0) put(0, l, V.x, W.x);
+      else {
+        put(k, l, V.x, -V.y);
+        if (2 * k != m) put(m - k, l, W.x, -W.y);
+      }
+    } else if (k == 0) {
+      put(0, l, (T)2 * V.x, (T)1.41421356237309504880 * W.x);
+    } else {
+      const cplx<T> c1 = cmul(ldg_c(t1 + k), V);
+      put(k, l, c1.x, -c1.y);
+      if (2 * k != m) {
+        const cplx<T> c2 = cmul(ldg_c(t1 + m - k), W);
+        put(m - k, l, c2.x, -c2.y);
+      }
+    }
+  }
+}
+
+// The slots to x lines, with the output modes of XformArgs (compiled per mode). sw: the
+// parts are traded; fd: the face-centred lines' slots, a value in part 0 of each.
+template <class D, class T, class TO, bool FWD, class Args, class Scale>
+__device__ __forceinline__ void x_store(const D& d, const Args& a, TO* out, size_t base, int live, const T* rS, int sw,
+                                        bool fd, bool scaled, Scale&& scale_of, T& tmax) {
+  const int n = d.n(), ls = d.ls(), bc = a.bc;
+  const T sg = (!FWD && bc == BC_DD) ? (T)-1 : (T)1;
+  const bool al = !((((uintptr_t)out) & (2 * sizeof(TO) - 1)) | (((uintptr_t)a.out2 | (uintptr_t)a.base32) & 7));
+  TO* dst = out + base;
+  const float* b32 = a.base32 ? a.base32 + base : nullptr;
+  float* o2 = a.out2 ? a.out2 + base : nullptr;
+  auto run = [&](auto kind, auto mode) {
+    constexpr int KIND = decltype(kind)::value, OM = decltype(mode)::value;
+    const SlotMap<D, KIND> map{d, bc};
+#pragma unroll 4
+    for (int idx = threadIdx.x; idx < live * (n >> 1); idx += blockDim.x) {
+      const int l = d.div_h(idx), e = 2 * (idx - l * (n >> 1));
+      int s0, c0, s1, c1;
+      if (fd) {
+        s0 = e;
+        s1 = e + 1;
+        c0 = c1 = 0;
+      } else if (FWD) {
+        map.spec_of(e, s0, c0, s1, c1);
+      } else {
+        map.phys_of(e, s0, c0, s1, c1);
+      }
+      T v0 = rS[2 * (s0 * ls + l) + (c0 ^ sw)], v1 = rS[2 * (s1 * ls + l) + (c1 ^ sw)];
+      if constexpr (!FWD && KIND == KIND_CT) v1 *= sg;
+      if (scaled) {
+        const T sc = scale_of(l);
+        v0 *= sc;
+        v1 *= sc;
+      }
+      const int g = 2 * idx;
+      if constexpr (sizeof(TO) == 8 && sizeof(T) == 4) {
+        const double w0 = widen_f32(v0), w1 = widen_f32(v1);
+        if constexpr (OM == row::OM_BASE) {
+          float f0, f1;
+          ld_pair(b32 + g, al, f0, f1);
+          st_pair(dst + g, al, widen_f32(f0) + w0, widen_f32(f1) + w1);
+        } else if constexpr (OM == row::OM_ACC) {
+          double b0, b1;
+          ld_pair(dst + g, al, b0, b1);
+          st_pair(dst + g, al, b0 + w0, b1 + w1);
+        } else if constexpr (OM == row::OM_STORE) {
+          st_pair(dst + g, al, w0, w1);
+        }
+        tmax = fmaxf(tmax, fmaxf(fabsf(v0), fabsf(v1)));
+        if (o2) st_pair(o2 + g, al, v0, v1);
+      } else if constexpr (OM == row::OM_ACC) {
+        TO b0, b1;
+        ld_pair(dst + g, al, b0, b1);
+        st_pair(dst + g, al, b0 + v0, b1 + v1);
+      } else {
+        st_pair(dst + g, al, v0, v1);
+      }
+    }
+  };
+  auto with_mode = [&](auto kind) {
+    if constexpr (!FWD && sizeof(TO) == 8 && sizeof(T) == 4) {
+      if (!out) return run(kind, std::integral_constant<int, row::OM_NONE>{});
+      if (b32) return run(kind, std::integral_constant<int, row::OM_BASE>{});
+    }
+    if (a.accumulate) run(kind, std::integral_constant<int, row::OM_ACC>{});
+    else run(kind, std::integral_constant<int, row::OM_STORE>{});
+  };
+  by_kind(bc, with_mode);
+}
+
+// max |value| of FP64 outputs (before widening: a 64-bit integer max would use the FP64 pipe)
+template <class T>
+__device__ __forceinline__ void amax_out(unsigned long long* amax, T tmax) {
+  if constexpr (sizeof(T) == 4) {
+    if (amax) {
+      for (int o = 16; o > 0; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+      const unsigned long long v = (unsigned long long)__double_as_longlong(st_cvt<double, T>::f(tmax));
+      if ((threadIdx.x & 31) == 0 && v) atomicMax(amax, v);
+    }
+  }
+}
 
 // Transforms tile `grp`; every thread of the CTA takes part; smem_raw holds
 // 2·(m + 1)·(L + 1) complex values (L = 1: 2·(m + 1)).
@@ -263,7 +466,7 @@ __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_
   TO* out = static_cast<TO*>(a.out);
   const int nx = a.nx, ny = a.ny, bc = a.bc;
   const bool iv = bc_iv(bc), fd = bc == BC_FD;
-  const SlotMap map{n, m, bc};
+  const DimRt dim{n, m, lgL, ls, tab.mg_m, tab.mg_h};
   const int tid = threadIdx.x, nt = blockDim.x;
 
   // ---- the tile: x: first element of row 0 of the group; y: column x0 of plane zb ----
@@ -297,26 +500,11 @@ __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_
       }
     }
   } else if (a.axis == 0) {
-    const bool al = !((uintptr_t)in & (2 * sizeof(TI) - 1));
-    const T sg = (FWD && bc == BC_DD) ? (T)-1 : (T)1;  // DST ordering: the odd elements change sign
-    for (int idx = tid; idx < live * m; idx += nt) {
-      const int l = div_mg(idx, tab.mg_m), e = 2 * (idx - l * m);
-      TI u0, u1;
-      ld_pair(in + base + (size_t)l * n + e, al, u0, u1);
-      T v0 = ld_cvt<T, TI>::f(u0), v1 = ld_cvt<T, TI>::f(u1);
-      if (fscale) {
-        const T sc = scale_of(l);
-        v0 *= sc;
-        v1 *= sc;
-      }
-      int s0, c0, s1, c1;
-      if (FWD) map.phys_of(e, s0, c0, s1, c1);
-      else map.spec_of(e, s0, c0, s1, c1);
-      rA[2 * (s0 * ls + l) + c0] = v0;
-      rA[2 * (s1 * ls + l) + c1] = sg * v1;
-    }
+    x_load<DimRt, T, TI, FWD>(dim, bc, in + base, live, rA, fscale, scale_of);
   } else {
     const T sc = fscale ? a.plane_scale[zb] : (T)1;
+    by_kind(bc, [&](auto kind) {
+    const SlotMap<DimRt, decltype(kind)::value> map{dim, bc};
 #pragma unroll 4
     for (int idx = tid; idx < (m << lgL); idx += nt) {
       const int l = idx & lm, p = idx >> lgL;
@@ -335,33 +523,13 @@ __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_
       }
       bufA[p * ls + l] = cplx<T>{v0, v1};
     }
+    });
   }
   __syncthreads();
 
-  // ---- 2. backward P, NN, DD: the pairs (k, m−k), in place, the parts traded for the
-  //         inverse FFT: Z_k = (V_k + conj V_{m−k})/2m + pb_k·(V_k − conj V_{m−k}),
-  //         pb_k = i·e^{+2πik/n}/2m; NN, DD: V_q = xb_q·(X_q − i X_{n−q}), xb_q = ½e^{+iπq/2n} ----
+  // ---- 2. backward P, NN, DD: the pairs (k, m−k), in place ----
   if (!FWD && !iv && !fd) {
-    const int np = m / 2 + 1;
-    const T s = tab.inv2m;
-    for (int idx = tid; idx < (np << lgL); idx += nt) {
-      const int l = idx & lm, k = idx >> lgL;
-      cplx<T>* A = bufA + k * ls + l;
-      cplx<T>* B = bufA + (k == 0 ? 0 : m - k) * ls + l;
-      const cplx<T> x = *A, y = *B;
-      cplx<T> V, W;
-      if (bc == BC_P) {
-        V = k == 0 ? cplx<T>{x.x, (T)0} : cplx<T>{x.x, -x.y};
-        W = k == 0 ? cplx<T>{x.y, (T)0} : cplx<T>{y.x, -y.y};
-      } else {
-        V = cmul(ldg_c(t1 + k), k == 0 ? cplx<T>{x.x, (T)0} : cplx<T>{x.x, -x.y});
-        W = cmul(ldg_c(t1 + m - k), k == 0 ? cplx<T>{x.y, -x.y} : cplx<T>{y.x, -y.y});
-      }
-      const cplx<T> Sm = cadd(V, conj_(W)), D = cmul(ldg_c(t0 + k), csub(V, conj_(W)));
-      const cplx<T> Zk = {s * Sm.x + D.x, s * Sm.y + D.y}, Zm = {s * Sm.x - D.x, D.y - s * Sm.y};
-      *A = {Zk.y, Zk.x};
-      if (k != 0 && 2 * k != m) *B = {Zm.y, Zm.x};
-    }
+    pairs_bwd(dim, bc, bufA, t0, t1, tab.inv2m, [&](int k, int l) { return bufA[k * ls + l]; });
     __syncthreads();
   }
 
@@ -392,7 +560,7 @@ __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_
 
   // ---- 4. post-processing in place (y, forward and DCT-IV: straight to the rows) ----
   T* rS = reinterpret_cast<T*>(src);
-  T tmax = (T)0;  // max |new value| before widening (a 64-bit integer max would use the FP64 pipe)
+  T tmax = (T)0;
   auto emit = [&](size_t g, T v) {  // one output value
     const TO x = st_cvt<TO, T>::f(v);
     if constexpr (sizeof(TO) == 8) {
@@ -414,10 +582,11 @@ __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_
   };
   const T yscale = (a.axis == 1 && bscale) ? a.plane_scale[zb] : (T)1;
   // the two values of slot k: kept in the slot (x), or written to their rows (y)
-  auto put = [&](int k, int l, T v0, T v1) {
+  auto put_as = [&](auto kind, int k, int l, T v0, T v1) {
     if (a.axis == 0) {
       src[k * ls + l] = cplx<T>{v0, v1};
     } else if (l < live) {
+      const SlotMap<DimRt, decltype(kind)::value> map{dim, bc};
       int e0, e1;
       if (FWD) map.spec(k, e0, e1);
       else map.phys(k, e0, e1);
@@ -443,35 +612,15 @@ __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_
     for (int idx = tid; idx < (m << lgL); idx += nt) {
       const int l = idx & lm, k = idx >> lgL;
       const cplx<T> c = cmul(ldg_c(t1 + k), src[k * ls + l]);
-      put(k, l, c.x, -c.y);
+      put_as(std::integral_constant<int, KIND_IV>{}, k, l, c.x, -c.y);
     }
     if (a.axis == 0) __syncthreads();
   } else if (FWD) {
-    // real DFT of the packed sequence: V_k = (Z_k + conj Z_{m−k})/2 + pf_k·(Z_k − conj Z_{m−k}),
-    // pf_k = −(i/2)e^{−2πik/n}; NN, DD: X_q = Re(xf_q V_q), X_{n−q} = −Im, xf_q = 2e^{−iπq/2n}
-    for (int idx = tid; idx < ((m / 2 + 1) << lgL); idx += nt) {
-      const int l = idx & lm, k = idx >> lgL;
-      const cplx<T> Zk = src[k * ls + l], Zm = src[(k == 0 ? 0 : m - k) * ls + l];
-      const cplx<T> Sm = cadd(Zk, conj_(Zm)), D = cmul(ldg_c(t0 + k), csub(Zk, conj_(Zm)));
-      const cplx<T> V = {(T)0.5 * Sm.x + D.x, (T)0.5 * Sm.y + D.y};
-      const cplx<T> W = {(T)0.5 * Sm.x - D.x, D.y - (T)0.5 * Sm.y};  // V_{m−k}
-      if (bc == BC_P) {
-        if (k == 0) put(0, l, V.x, W.x);
-        else {
-          put(k, l, V.x, -V.y);
-          if (2 * k != m) put(m - k, l, W.x, -W.y);
-        }
-      } else if (k == 0) {
-        put(0, l, (T)2 * V.x, (T)1.41421356237309504880 * W.x);
-      } else {
-        const cplx<T> c1 = cmul(ldg_c(t1 + k), V);
-        put(k, l, c1.x, -c1.y);
-        if (2 * k != m) {
-          const cplx<T> c2 = cmul(ldg_c(t1 + m - k), W);
-          put(m - k, l, c2.x, -c2.y);
-        }
-      }
-    }
+    auto pairs = [&](auto kind) {
+      pairs_fwd(dim, bc, src, t0, t1, [&](int k, int l, T v0, T v1) { put_as(kind, k, l, v0, v1); });
+    };
+    if (bc == BC_P) pairs(std::integral_constant<int, KIND_P>{});
+    else pairs(std::integral_constant<int, KIND_CT>{});
     if (a.axis == 0) __syncthreads();
   }
 
@@ -479,56 +628,15 @@ __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_
   // backward P, NN, DD: the FFT's parts are still traded (part c of a slot is 1 − c)
   const int sw = (!FWD && !iv && !fd) ? 1 : 0;
   if (a.axis == 0) {
-    const T sg = (!FWD && bc == BC_DD) ? (T)-1 : (T)1;
-    const bool al = !((((uintptr_t)out) & (2 * sizeof(TO) - 1)) | (((uintptr_t)a.out2 | (uintptr_t)a.base32) & 7));
-    for (int idx = tid; idx < live * (n >> 1); idx += nt) {
-      const int l = div_mg(idx, tab.mg_h), e = 2 * (idx - l * (n >> 1));
-      int s0, c0, s1, c1;
-      if (fd) {
-        s0 = e;
-        s1 = e + 1;
-        c0 = c1 = 0;
-      } else if (FWD) {
-        map.spec_of(e, s0, c0, s1, c1);
-      } else {
-        map.phys_of(e, s0, c0, s1, c1);
-      }
-      T v0 = rS[2 * (s0 * ls + l) + (c0 ^ sw)], v1 = sg * rS[2 * (s1 * ls + l) + (c1 ^ sw)];
-      if (bscale) {
-        const T sc = scale_of(l);
-        v0 *= sc;
-        v1 *= sc;
-      }
-      const size_t g = base + (size_t)l * n + e;
-      if constexpr (sizeof(TO) == 8 && sizeof(T) == 4) {
-        if (out) {
-          double b0 = 0.0, b1 = 0.0;
-          const double w0 = widen_f32(v0), w1 = widen_f32(v1);
-          if (a.base32) {
-            float f0, f1;
-            ld_pair(a.base32 + g, al, f0, f1);
-            b0 = widen_f32(f0);
-            b1 = widen_f32(f1);
-          } else if (a.accumulate) {
-            ld_pair(out + g, al, b0, b1);
-          }
-          const bool add = a.base32 || a.accumulate;
-          st_pair(out + g, al, add ? b0 + w0 : w0, add ? b1 + w1 : w1);
-        }
-        tmax = fmaxf(tmax, fmaxf(fabsf(v0), fabsf(v1)));
-        if (a.out2) st_pair(a.out2 + g, al, v0, v1);
-      } else {
-        TO b0 = (TO)0, b1 = (TO)0;
-        if (a.accumulate) ld_pair(out + g, al, b0, b1);
-        st_pair(out + g, al, a.accumulate ? b0 + v0 : v0, a.accumulate ? b1 + v1 : v1);
-      }
-    }
+    x_store<DimRt, T, TO, FWD>(dim, a, out, base, live, rS, sw, fd, bscale, scale_of, tmax);
   } else if (fd) {
     for (int idx = tid; idx < (n << lgL); idx += nt) {
       const int l = idx & lm, e = idx >> lgL;
       if (l < live) emit(base + (size_t)(e * nx) + l, rS[2 * (e * ls + l)] * yscale);
     }
   } else if (!FWD && !iv) {
+    by_kind(bc, [&](auto kind) {
+    const SlotMap<DimRt, decltype(kind)::value> map{dim, bc};
     for (int idx = tid; idx < (m << lgL); idx += nt) {
       const int l = idx & lm, p = idx >> lgL;
       if (l >= live) continue;
@@ -539,14 +647,9 @@ __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_
       emit(base + (size_t)(e0 * nx) + l, v0 * yscale);
       emit(base + (size_t)(e1 * nx) + l, v1 * yscale);
     }
+    });
   }
-  if constexpr (sizeof(TO) == 8 && sizeof(T) == 4) {
-    if (a.amax) {
-      for (int o = 16; o > 0; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
-      const unsigned long long amax = (unsigned long long)__double_as_longlong(st_cvt<double, T>::f(tmax));
-      if ((threadIdx.x & 31) == 0 && amax) atomicMax(a.amax, amax);
-    }
-  }
+  if constexpr (sizeof(TO) == 8) amax_out(a.amax, tmax);
 }
 
 }  // namespace ps

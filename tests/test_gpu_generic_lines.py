@@ -1,4 +1,4 @@
-"""The generic line transforms at the edges of their tiles.
+"""The line transforms of lengths that are no power of two, at the edges of their tiles.
 
 Lines whose half length is not a power of two, or that sit in planes whose n_x is no multiple
 of a tile of lines, run in one kernel with run-time radices (16, 9, 8, 6, 4, 3, 2). The cases
@@ -52,3 +52,26 @@ def test_generic_lines_match_oracle(lib, nx, ny, nz, bx, by):
                           ("fp32_refine", 1e-9, dict(rtol=1e-10, max_iter=6))):
         p = _solve(lib, f, dx, dy, zf, bcs, precision=prec, **kw)
         assert np.abs(p - q).max() <= tol * scale, (prec, np.abs(p - q).max() / scale)
+
+
+# half lengths with a compile-time kernel, paired so that each runs on x and on y; n_z gives
+# every SM a tile (the rule of the dispatch), the last tiles of a plane are partial
+HALF = [(486, 16), (432, 18), (384, 24), (324, 27), (288, 32), (243, 36), (216, 48), (192, 54), (162, 72),
+        (144, 81), (108, 96)]
+BCS = ["P", "NN", "DD", "ND", "DN"]
+
+
+@pytest.mark.parametrize("mx,my", HALF + [(b, a) for a, b in HALF])
+def test_compile_time_lines_match_oracle(lib, mx, my):
+    nx, ny, nz = 2 * mx, 2 * my, 77
+    zf = synth.tanh_faces(nz, 1.0, 1.5)
+    dx, dy = 2.0 / nx, 1.0 / ny
+    f = synth.uniform_noise((nz, ny, nx), seed=nx + ny, remove_mean=False)
+    i = HALF.index((max(mx, my), min(mx, my)))
+    for bx, by, prec, tol, kw in ((BCS[i % 5], BCS[(i + 1) % 5], "fp32", 5e-5, {}),
+                                  (BCS[(i + 2) % 5], BCS[(i + 4) % 5], "fp32_refine", 1e-9,
+                                   dict(rtol=1e-10, max_iter=6))):
+        bcs = (bx, by, "DD")
+        q = S.solve(f, dx, dy, zf, *bcs)
+        p = _solve(lib, f, dx, dy, zf, bcs, precision=prec, **kw)
+        assert np.abs(p - q).max() <= tol * np.abs(q).max(), (prec, bcs, np.abs(p - q).max() / np.abs(q).max())
