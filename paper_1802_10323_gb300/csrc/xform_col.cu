@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(CShape<M, CW>::NT, sizeof(T) == 4 ? 1024 / CSh
   cplx<T>* ptw = stw + M;                               // e^{−2πik/n}, k ≤ M
   cplx<T>* xtw = ptw + (M + 1);                         // NN/DD: e^{−iπq/2n}, q < n; ND: pre, post
   cplx<T>* buf = reinterpret_cast<cplx<T>*>(smem_raw + fast_table_bytes<T, M>(a.bc));  // [M][CW]
-  load_line_tables<T, M>(a.tw, a.bc, stw);
+  load_line_tables<T, M, FWD>(a.tw, a.bc, stw);
   pdl_wait();
   if (a.skip && *a.skip) return;
   const int ntiles = a.nz * (a.nx / CW);

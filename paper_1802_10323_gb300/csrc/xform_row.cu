@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(32 * WARPS, sizeof(T) == 4 ? (M >= 512 ? 3 : 4
   cplx<T>* ptw = stw + M;
   cplx<T>* xtw = ptw + (M + 1);
   cplx<T>* bufs = reinterpret_cast<cplx<T>*>(smem_raw + fast_table_bytes<T, M>(a.bc));
-  load_line_tables<T, M>(a.tw, a.bc, stw);
+  load_line_tables<T, M, FWD>(a.tw, a.bc, stw);
   pdl_wait();
   if (a.skip && *a.skip) return;
   __syncthreads();  // the only block-wide barrier: tables ready

@@ -13,21 +13,48 @@ namespace ps {
 
 // Twiddle tables of one axis into shared memory at stw: ω_M^t (t < M), the
 // real-FFT split factors (M + 1) and the BC factors (NN/DD: n; ND: 2·M).
-template <class T, int M>
+// The halves of the split, the 2 of the cosine outputs and the 1/M and 1/n of the
+// backward transform are powers of two and sit in the factors that multiply every value
+// anyway (or in a fused multiply-add with the split's sum, split_scale): the results
+// keep their bits, and the FP64 passes, which the FP64 pipe bounds, lose a quarter of
+// their arithmetic outside the FFT stages (NN pair of wavenumbers, forward 32 → 20
+// instructions, backward 36 → 20). FP64 256³ (DD, ND, NN) 2945 → 2647 µs; FP32 passes
+// are bound by memory and keep their time.
+template <class T, int M, bool FWD>
 __device__ __forceinline__ void load_line_tables(const cplx<T>* tw, int bc, cplx<T>* stw) {
   constexpr int N = 2 * M;
+  constexpr T half = (T)0.5, inv_m = (T)1 / (T)M;  // exact
   cplx<T>* ptw = stw + M;
   cplx<T>* xtw = ptw + (M + 1);
   for (int i = threadIdx.x; i < M; i += blockDim.x) stw[i] = tw[16 * i];
-  for (int i = threadIdx.x; i <= M; i += blockDim.x) ptw[i] = tw[8 * i];
+  const T fs = bc == BC_P ? (FWD ? half : half * inv_m) : (T)1;
+  for (int i = threadIdx.x; i <= M; i += blockDim.x) ptw[i] = cscale(tw[8 * i], fs);
   if (bc == BC_NN || bc == BC_DD) {
-    for (int i = threadIdx.x; i < N; i += blockDim.x) xtw[i] = tw[2 * i];
+    for (int i = threadIdx.x; i < N; i += blockDim.x)
+      xtw[i] = FWD ? tw[2 * i] : cscale(tw[2 * i], half * half * inv_m);
   } else if (bc_iv(bc)) {
     for (int i = threadIdx.x; i < M; i += blockDim.x) {
       xtw[i] = tw[4 * i];
-      xtw[M + i] = tw[4 * i + 1];
+      xtw[M + i] = cscale(tw[4 * i + 1], FWD ? (T)2 : half * inv_m);
     }
   }
+}
+
+// The two wavenumbers of a pair from (or to) its even and odd parts e, o (o already
+// multiplied by its table factor): h·e ± o with the factor h of periodic lines, which
+// have no other table to hold it (h = 1 and a plain sum otherwise).
+template <class T>
+__device__ __forceinline__ cplx<T> split_add(cplx<T> e, cplx<T> o, T h) {
+  return {fma(h, e.x, o.x), fma(h, e.y, o.y)};
+}
+template <class T>
+__device__ __forceinline__ cplx<T> split_sub(cplx<T> e, cplx<T> o, T h) {
+  return {fma(h, e.x, -o.x), fma(h, e.y, -o.y)};
+}
+// h of a line's split (see above).
+template <class T, int M, bool FWD>
+__device__ __forceinline__ T split_scale(int bc) {
+  return bc == BC_P ? (FWD ? (T)0.5 : (T)0.5 / (T)M) : (T)1;
 }
 
 namespace row {
@@ -75,7 +102,7 @@ struct LaneSlots {
 
 // One line (two for M = 64, half a warp each) of the x transform: the warp's
 // exchange buffers at bufs, tables in shared memory, the first line index l0.
-// tmax accumulates max |FP64 output| (before widening) for the caller's reduction.
+// tmax accumulates max |FP64 output| (before widening; an FP64 transform only when asked, on its own pipe) for the caller's reduction.
 template <class T, class TI, class TO, int M, bool FWD, int OM>
 __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* stw, const cplx<T>* ptw,
                                          const cplx<T>* xtw, cplx<T>* bufs, int l0, T& tmax) {
@@ -97,7 +124,9 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
   const size_t base = (size_t)(live ? line : l0) * N;
   const TI* src = in + base;
   TO* dst = out + base;
-  const T s = a.plane_scale ? a.plane_scale[(live ? line : l0) / ny] : (T)1;
+  const bool scaled = a.plane_scale != nullptr;
+  const T s = scaled ? a.plane_scale[(live ? line : l0) / ny] : (T)1;
+  const T h = split_scale<T, M, FWD>(bc);
   cplx<T> v[E];
   if (FWD) {
     // ---- gather the first-stage operands from the line ----
@@ -107,7 +136,7 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
       for (int si = 0; si < E; ++si) {
         const int p = t + (si / R0) * TPL + (si % R0) * (M / R0);
         const vec<TI, 2> x = *reinterpret_cast<const vec<TI, 2>*>(src + 2 * p);
-        v[si] = {in_cvt<T>(x.v[0]) * s, in_cvt<T>(x.v[1]) * s};
+        v[si] = {in_cvt<T>(x.v[0]), in_cvt<T>(x.v[1])};
       }
     } else if (bc_iv(bc)) {
       // z_p = (x_{2p}, x_{n−1−2p})·e^{−iπp/n}; x_{n−1−2p} = x_{2p'+1} of p' = M−1−p
@@ -116,8 +145,8 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
       for (int si = 0; si < E; ++si) {
         const int p = t + (si / R0) * TPL + (si % R0) * (M / R0);
         const vec<TI, 2> x = *reinterpret_cast<const vec<TI, 2>*>(src + 2 * p);
-        v[si].x = in_cvt<T>(x.v[0]) * s;
-        const T odd = in_cvt<T>(x.v[1]) * s;
+        v[si].x = in_cvt<T>(x.v[0]);
+        const T odd = in_cvt<T>(x.v[1]);
         v[E - 1 - si].y = __shfl_sync(full, odd, mate);
       }
       if (bc == BC_DN) {
@@ -132,7 +161,7 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
     } else {
       // z_p = (v_{2p}, v_{2p+1}) with v_j = x_{2j} (j < M), ±x_{2n−1−2j} (j ≥ M, − for DD);
       // the 4-vector at 4p (p < M/2) is (z_p.x, z_{p'}.y, z_p.y, z_{p'}.x), p' = M−1−p
-      const T sg = (bc == BC_DD) ? (T)-1 : (T)1;
+      const bool neg = (bc == BC_DD);
 #pragma unroll
       for (int si = 0; si < E; ++si) {
         if ((si % R0) >= R0 / 2) continue;
@@ -141,19 +170,23 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
         if constexpr (sizeof(TI) == 4) {
           const vec<TI, 4> q = *reinterpret_cast<const vec<TI, 4>*>(src + 4 * p);
 #pragma unroll
-          for (int u = 0; u < 4; ++u) x[u] = in_cvt<T>(q.v[u]) * s;
+          for (int u = 0; u < 4; ++u) x[u] = in_cvt<T>(q.v[u]);
         } else {
           const vec<TI, 2> q0 = *reinterpret_cast<const vec<TI, 2>*>(src + 4 * p);
           const vec<TI, 2> q1 = *reinterpret_cast<const vec<TI, 2>*>(src + 4 * p + 2);
-          x[0] = in_cvt<T>(q0.v[0]) * s;
-          x[1] = in_cvt<T>(q0.v[1]) * s;
-          x[2] = in_cvt<T>(q1.v[0]) * s;
-          x[3] = in_cvt<T>(q1.v[1]) * s;
+          x[0] = in_cvt<T>(q0.v[0]);
+          x[1] = in_cvt<T>(q0.v[1]);
+          x[2] = in_cvt<T>(q1.v[0]);
+          x[3] = in_cvt<T>(q1.v[1]);
         }
         v[si] = {x[0], x[2]};
         const T ry = __shfl_sync(full, x[1], mate), rx = __shfl_sync(full, x[3], mate);
-        v[E - 1 - si] = {sg * rx, sg * ry};
+        v[E - 1 - si] = neg ? cplx<T>{-rx, -ry} : cplx<T>{rx, ry};
       }
+    }
+    if (scaled) {
+#pragma unroll
+      for (int si = 0; si < E; ++si) v[si] = cscale(v[si], s);
     }
     fast::fft_stages<T, M, false, 0, 1>(v, lc, stw, t);
     if constexpr (TPL == 32) {
@@ -172,8 +205,8 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
         for (int j = 0; j < E; ++j) {
           const int k = t + 32 * j;
           const cplx<T> c = cmul(xtw[M + k], v[LS::sout(j)]);
-          Y(2 * k, (T)2 * c.x);
-          Y(N - 1 - 2 * k, (T)-2 * c.y);
+          Y(2 * k, c.x);
+          Y(N - 1 - 2 * k, -c.y);
         }
       } else {
         const int pl = (32 - t) & 31;
@@ -181,10 +214,10 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
         auto OUTQ = [&](int q, T val) { Y(rev ? (N - 1 - q) : q, val); };
         // outputs of k (and of M − k unless k = 0 or 2k = M) from Z_k and Z_{M−k}
         auto pair_out = [&](int k, cplx<T> Zk, cplx<T> Zmk) {
-          const cplx<T> Ek = cscale(cadd(Zk, conj_(Zmk)), (T)0.5);
-          const cplx<T> Ok = cscale(mul_mi(csub(Zk, conj_(Zmk))), (T)0.5);
+          const cplx<T> Ek = cadd(Zk, conj_(Zmk));
+          const cplx<T> Ok = mul_mi(csub(Zk, conj_(Zmk)));
           const cplx<T> B = cmul(ptw[k], Ok);
-          const cplx<T> Vk = cadd(Ek, B), Vmk = conj_(csub(Ek, B));
+          const cplx<T> Vk = split_add(Ek, B, h), Vmk = conj_(split_sub(Ek, B, h));
           if (bc == BC_P) {
             if (k == 0) {
               Y(0, Vk.x);
@@ -198,16 +231,16 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
               }
             }
           } else if (k == 0) {
-            OUTQ(0, (T)2 * Vk.x);
-            OUTQ(M, (T)1.41421356237309504880 * Vmk.x);
+            OUTQ(0, Vk.x);
+            OUTQ(M, (T)0.70710678118654752440 * Vmk.x);
           } else {
             const cplx<T> c1 = cmul(xtw[k], Vk);
-            OUTQ(k, (T)2 * c1.x);
-            OUTQ(N - k, (T)-2 * c1.y);
+            OUTQ(k, c1.x);
+            OUTQ(N - k, -c1.y);
             if (2 * k != M) {
               const cplx<T> c2 = cmul(xtw[M - k], Vmk);
-              OUTQ(M - k, (T)2 * c2.x);
-              OUTQ(M + k, (T)-2 * c2.y);
+              OUTQ(M - k, c2.x);
+              OUTQ(M + k, -c2.y);
             }
           }
         };
@@ -239,8 +272,8 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
         for (int i = 0; i < E; ++i) {
           const int k = t + i * TPL;
           const cplx<T> c = cmul(xtw[M + k], lc[cpad(k)]);
-          Y(2 * k, (T)2 * c.x);
-          Y(N - 1 - 2 * k, (T)-2 * c.y);
+          Y(2 * k, c.x);
+          Y(N - 1 - 2 * k, -c.y);
         }
       } else {
         constexpr int NP = (M / 2) / TPL + 1;
@@ -249,10 +282,10 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
           const int k = t + i * TPL;
           if (k > M / 2) break;
           const cplx<T> Zk = lc[cpad(k)], Zmk = lc[cpad(k == 0 ? 0 : M - k)];
-          const cplx<T> Ek = cscale(cadd(Zk, conj_(Zmk)), (T)0.5);
-          const cplx<T> Ok = cscale(mul_mi(csub(Zk, conj_(Zmk))), (T)0.5);
+          const cplx<T> Ek = cadd(Zk, conj_(Zmk));
+          const cplx<T> Ok = mul_mi(csub(Zk, conj_(Zmk)));
           const cplx<T> B = cmul(ptw[k], Ok);
-          const cplx<T> Vk = cadd(Ek, B), Vmk = conj_(csub(Ek, B));
+          const cplx<T> Vk = split_add(Ek, B, h), Vmk = conj_(split_sub(Ek, B, h));
           if (bc == BC_P) {
             if (k == 0) {
               Y(0, Vk.x);
@@ -269,16 +302,16 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
             const bool rev = (bc == BC_DD);
             auto OUTQ = [&](int q, T val) { Y(rev ? (N - 1 - q) : q, val); };
             if (k == 0) {
-              OUTQ(0, (T)2 * Vk.x);
-              OUTQ(M, (T)1.41421356237309504880 * Vmk.x);
+              OUTQ(0, Vk.x);
+              OUTQ(M, (T)0.70710678118654752440 * Vmk.x);
             } else {
               const cplx<T> c1 = cmul(xtw[k], Vk);
-              OUTQ(k, (T)2 * c1.x);
-              OUTQ(N - k, (T)-2 * c1.y);
+              OUTQ(k, c1.x);
+              OUTQ(N - k, -c1.y);
               if (2 * k != M) {
                 const cplx<T> c2 = cmul(xtw[M - k], Vmk);
-                OUTQ(M - k, (T)2 * c2.x);
-                OUTQ(M + k, (T)-2 * c2.y);
+                OUTQ(M - k, c2.x);
+                OUTQ(M + k, -c2.y);
               }
             }
           }
@@ -329,7 +362,7 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
             const T x0 = X(qx(k)), x1 = (k == 0) ? (T)0 : X(qx(N - k));
             cplx<T> w = xtw[k];
             w.y = -w.y;
-            Vv[j] = cscale(cmul(w, cplx<T>{x0, -x1}), (T)0.5);
+            Vv[j] = cmul(w, cplx<T>{x0, -x1});
           }
         }
         // V_M, the partner of k = 0 (lane 0)
@@ -340,7 +373,7 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
           const T xm = X(qx(M));
           cplx<T> w = xtw[M];
           w.y = -w.y;
-          VM = cscale(cmul(w, cplx<T>{xm, -xm}), (T)0.5);
+          VM = cmul(w, cplx<T>{xm, -xm});
         }
         const int pl = (32 - t) & 31;
 #pragma unroll
@@ -348,11 +381,11 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
           const int k = t + 32 * j;
           cplx<T> Vm = {__shfl_sync(full, Vv[E - 1 - j].x, pl), __shfl_sync(full, Vv[E - 1 - j].y, pl)};
           if (t == 0) Vm = (j == 0) ? VM : Vv[(E - j) % E];
-          const cplx<T> Ek = cscale(cadd(Vv[j], conj_(Vm)), (T)0.5);
+          const cplx<T> Ek = cadd(Vv[j], conj_(Vm));
           cplx<T> wn = ptw[k];
           wn.y = -wn.y;
-          const cplx<T> Ok = cscale(cmul(csub(Vv[j], conj_(Vm)), wn), (T)0.5);
-          v[LS::sin_(j)] = cadd(Ek, mul_i(Ok));
+          const cplx<T> Ok = cmul(csub(Vv[j], conj_(Vm)), wn);
+          v[LS::sin_(j)] = split_add(Ek, mul_i(Ok), h);
         }
       }
     } else {
@@ -409,17 +442,17 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
           } else {
             cplx<T> w = xtw[k];
             w.y = -w.y;
-            Vk = cscale(cmul(w, cplx<T>{xv[i][0], -xv[i][1]}), (T)0.5);
+            Vk = cmul(w, cplx<T>{xv[i][0], -xv[i][1]});
             cplx<T> w2 = xtw[M - k];
             w2.y = -w2.y;
-            Vm = cscale(cmul(w2, cplx<T>{xv[i][2], -xv[i][3]}), (T)0.5);
+            Vm = cmul(w2, cplx<T>{xv[i][2], -xv[i][3]});
           }
-          const cplx<T> Ek = cscale(cadd(Vk, conj_(Vm)), (T)0.5);
+          const cplx<T> Ek = cadd(Vk, conj_(Vm));
           cplx<T> wn = ptw[k];
           wn.y = -wn.y;
-          const cplx<T> Ok = cscale(cmul(csub(Vk, conj_(Vm)), wn), (T)0.5);
-          if (k < M) lc[cpad(k)] = cadd(Ek, mul_i(Ok));
-          if (k != 0 && 2 * k != M) lc[cpad(M - k)] = cadd(conj_(Ek), mul_i(conj_(Ok)));
+          const cplx<T> Ok = cmul(csub(Vk, conj_(Vm)), wn);
+          if (k < M) lc[cpad(k)] = split_add(Ek, mul_i(Ok), h);
+          if (k != 0 && 2 * k != M) lc[cpad(M - k)] = split_add(conj_(Ek), mul_i(conj_(Ok)), h);
         }
       }
       __syncwarp();
@@ -448,12 +481,12 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
       }
 #pragma unroll
       for (int u = 0; u < NV; ++u) {
-        o2.v[u] = val[u] * s;
+        o2.v[u] = val[u];
         const TO x = st_cvt<TO, T>::f(o2.v[u]);
         if constexpr (OM == OM_ACC || (F64OUT && OM == OM_BASE)) o.v[u] = o.v[u] + x;
         else o.v[u] = x;
         if constexpr (sizeof(TO) == 8)
-          if (live) tmax = fmax(tmax, fabs(o2.v[u]));
+          if (live && (sizeof(T) == 4 || a.amax)) tmax = fmax(tmax, fabs(o2.v[u]));
       }
       if (live) {
         if constexpr (OM != OM_NONE) *reinterpret_cast<vec<TO, NV>*>(dst + i0) = o;
@@ -463,25 +496,27 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
     };
     using two = std::integral_constant<int, 2>;
     using four = std::integral_constant<int, 4>;
-    const T inv_m = (T)1 / (T)M;
+    if (scaled) {
+#pragma unroll
+      for (int si = 0; si < E; ++si) v[si] = cscale(v[si], s);
+    }
     if (bc == BC_P) {
 #pragma unroll
       for (int si = 0; si < E; ++si) {
         const int k = t + (si / RL) * TPL + (si % RL) * (M / RL);
-        const T val[2] = {v[si].x * inv_m, v[si].y * inv_m};
+        const T val[2] = {v[si].x, v[si].y};
         put(2 * k, val, two{});
       }
     } else if (bc_iv(bc)) {
-      // output 2k = Re(c_k)/n, output n−1−2k = −Im(c_k)/n with c_k = e^{...}·z_k;
-      // the pair (2k, 2k+1) takes −Im(c_{k'})/n of k' = M−1−k from the mirrored slot
+      // output 2k = Re(c_k), output n−1−2k = −Im(c_k) with c_k = e^{...}·z_k/n;
+      // the pair (2k, 2k+1) takes −Im(c_{k'}) of k' = M−1−k from the mirrored slot
       // (DN, the reversed line: the two outputs of each k trade places)
-      const T inv_n = (T)1 / (T)N;
       T re[E], im[E];
 #pragma unroll
       for (int si = 0; si < E; ++si) {
         const int k = t + (si / RL) * TPL + (si % RL) * (M / RL);
         const cplx<T> c = cmul(xtw[M + k], v[si]);
-        const T A = c.x * inv_n, B = -c.y * inv_n;
+        const T A = c.x, B = -c.y;
         re[si] = (bc == BC_DN) ? B : A;
         im[si] = (bc == BC_DN) ? A : B;
       }
@@ -495,14 +530,14 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
       // z_k → outputs (i0, i1) = (4k, 4k+2) for k < M/2 and the odd (2n−1−4k, 2n−3−4k)
       // for k ≥ M/2 (negated for DD): the 4-vector at 4k (k < M/2) is
       // (z_k.x, ±z_{k'}.y, z_k.y, ±z_{k'}.x), k' = M−1−k
-      const T sg = (bc == BC_DD) ? (T)-1 : (T)1;
+      const bool neg = (bc == BC_DD);
 #pragma unroll
       for (int si = 0; si < E; ++si) {
         const int j = E - 1 - si;  // every lane hands its mirrored slot to its mate
         const T hy = __shfl_sync(full, v[j].y, mate), hx = __shfl_sync(full, v[j].x, mate);
         if ((si % RL) >= RL / 2) continue;
         const int k = t + (si / RL) * TPL + (si % RL) * (M / RL);
-        const T val[4] = {v[si].x * inv_m, sg * hy * inv_m, v[si].y * inv_m, sg * hx * inv_m};
+        const T val[4] = {v[si].x, neg ? -hy : hy, v[si].y, neg ? -hx : hx};
         put(4 * k, val, four{});
       }
     }
@@ -645,7 +680,9 @@ __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* st
   // row offsets fit in 32 bits (n_y·n_x ≤ 2^20)
   auto X = [&](int q) { return src[q * sstr]; };
   auto Y = [&](int q, T val) { dst[q * nx] = val; };
-  const T s = a.plane_scale ? a.plane_scale[zb] : (T)1;
+  const bool scaled = a.plane_scale != nullptr;
+  const T s = scaled ? a.plane_scale[zb] : (T)1;
+  const T h = split_scale<T, M, FWD>(bc);
   cplx<T> v[E];
   __syncthreads();  // tables ready; the previous tile's buffer reads are done
   if (FWD) {
@@ -668,7 +705,11 @@ __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* st
         }
         z = {v0, v1};
       }
-      v[r] = cscale(z, s);
+      v[r] = z;
+    }
+    if (scaled) {
+#pragma unroll
+      for (int r = 0; r < E; ++r) v[r] = cscale(v[r], s);
     }
     fft_col<T, M, CW, false, 0, 1>(v, buf, stw, b, c);
     // ---- post-processing: pair k with M − k through the buffer, rows out ----
@@ -683,8 +724,8 @@ __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* st
       for (int i = 0; i < E; ++i) {
         const int k = b + i * TPL;
         const cplx<T> cc = cmul(xtw[M + k], buf[k * CW + c]);
-        Y(2 * k, (T)2 * cc.x);
-        Y(N - 1 - 2 * k, (T)-2 * cc.y);
+        Y(2 * k, cc.x);
+        Y(N - 1 - 2 * k, -cc.y);
       }
     } else {
       constexpr int NP = (M / 2) / TPL + 1;
@@ -693,10 +734,10 @@ __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* st
         const int k = b + i * TPL;
         if (k > M / 2) break;
         const cplx<T> Zk = buf[k * CW + c], Zmk = buf[(k == 0 ? 0 : M - k) * CW + c];
-        const cplx<T> Ek = cscale(cadd(Zk, conj_(Zmk)), (T)0.5);
-        const cplx<T> Ok = cscale(mul_mi(csub(Zk, conj_(Zmk))), (T)0.5);
+        const cplx<T> Ek = cadd(Zk, conj_(Zmk));
+        const cplx<T> Ok = mul_mi(csub(Zk, conj_(Zmk)));
         const cplx<T> B = cmul(ptw[k], Ok);
-        const cplx<T> Vk = cadd(Ek, B), Vmk = conj_(csub(Ek, B));
+        const cplx<T> Vk = split_add(Ek, B, h), Vmk = conj_(split_sub(Ek, B, h));
         if (bc == BC_P) {
           if (k == 0) {
             Y(0, Vk.x);
@@ -713,16 +754,16 @@ __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* st
           const bool rev = (bc == BC_DD);
           auto OUTQ = [&](int q, T val) { Y(rev ? (N - 1 - q) : q, val); };
           if (k == 0) {
-            OUTQ(0, (T)2 * Vk.x);
-            OUTQ(M, (T)1.41421356237309504880 * Vmk.x);
+            OUTQ(0, Vk.x);
+            OUTQ(M, (T)0.70710678118654752440 * Vmk.x);
           } else {
             const cplx<T> c1 = cmul(xtw[k], Vk);
-            OUTQ(k, (T)2 * c1.x);
-            OUTQ(N - k, (T)-2 * c1.y);
+            OUTQ(k, c1.x);
+            OUTQ(N - k, -c1.y);
             if (2 * k != M) {
               const cplx<T> c2 = cmul(xtw[M - k], Vmk);
-              OUTQ(M - k, (T)2 * c2.x);
-              OUTQ(M + k, (T)-2 * c2.y);
+              OUTQ(M - k, c2.x);
+              OUTQ(M + k, -c2.y);
             }
           }
         }
@@ -775,17 +816,17 @@ __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* st
         } else {
           cplx<T> w = xtw[k];
           w.y = -w.y;
-          Vk = cscale(cmul(w, cplx<T>{xv[i][0], -xv[i][1]}), (T)0.5);
+          Vk = cmul(w, cplx<T>{xv[i][0], -xv[i][1]});
           cplx<T> w2 = xtw[M - k];
           w2.y = -w2.y;
-          Vm = cscale(cmul(w2, cplx<T>{xv[i][2], -xv[i][3]}), (T)0.5);
+          Vm = cmul(w2, cplx<T>{xv[i][2], -xv[i][3]});
         }
-        const cplx<T> Ek = cscale(cadd(Vk, conj_(Vm)), (T)0.5);
+        const cplx<T> Ek = cadd(Vk, conj_(Vm));
         cplx<T> wn = ptw[k];
         wn.y = -wn.y;
-        const cplx<T> Ok = cscale(cmul(csub(Vk, conj_(Vm)), wn), (T)0.5);
-        if (k < M) buf[k * CW + c] = cadd(Ek, mul_i(Ok));
-        if (k != 0 && 2 * k != M) buf[(M - k) * CW + c] = cadd(conj_(Ek), mul_i(conj_(Ok)));
+        const cplx<T> Ok = cmul(csub(Vk, conj_(Vm)), wn);
+        if (k < M) buf[k * CW + c] = split_add(Ek, mul_i(Ok), h);
+        if (k != 0 && 2 * k != M) buf[(M - k) * CW + c] = split_add(conj_(Ek), mul_i(conj_(Ok)), h);
       }
     }
     __syncthreads();
@@ -794,7 +835,10 @@ __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* st
     if (bc_iv(bc)) fft_col<T, M, CW, false, 0, 1>(v, buf, stw, b, c);
     else fft_col<T, M, CW, true, 0, 1>(v, buf, stw, b, c);
     // ---- backward post-processing straight from the last stage to the rows ----
-    const T inv_m = (T)1 / (T)M;
+    if (scaled) {
+#pragma unroll
+      for (int r = 0; r < E; ++r) v[r] = cscale(v[r], s);
+    }
 #pragma unroll
     for (int q = 0; q < E / RL; ++q) {
 #pragma unroll
@@ -803,7 +847,7 @@ __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* st
         const cplx<T> zk = v[q * RL + r];
         if (bc_iv(bc)) {
           const cplx<T> cc = cmul(xtw[M + k], zk);
-          const T A = cc.x * ((T)1 / (T)N) * s, B = -cc.y * ((T)1 / (T)N) * s;
+          const T A = cc.x, B = -cc.y;
           if (bc == BC_DN) {
             Y(2 * k, B);
             Y(N - 1 - 2 * k, A);
@@ -812,13 +856,13 @@ __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* st
             Y(N - 1 - 2 * k, B);
           }
         } else if (bc == BC_P) {
-          Y(2 * k, zk.x * inv_m * s);
-          Y(2 * k + 1, zk.y * inv_m * s);
+          Y(2 * k, zk.x);
+          Y(2 * k + 1, zk.y);
         } else {
           const int j0 = 2 * k, j1 = 2 * k + 1;
           const int i0 = j0 < M ? 2 * j0 : 2 * N - 1 - 2 * j0;
           const int i1 = j1 < M ? 2 * j1 : 2 * N - 1 - 2 * j1;
-          T v0 = zk.x * inv_m * s, v1 = zk.y * inv_m * s;
+          T v0 = zk.x, v1 = zk.y;
           if (bc == BC_DD) {
             if (i0 & 1) v0 = -v0;
             if (i1 & 1) v1 = -v1;
