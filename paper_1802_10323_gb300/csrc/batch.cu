@@ -307,7 +307,7 @@ __device__ __forceinline__ int ld_relaxed(const int* p) {
 // memory latencies (~0.7 µs each): an entry carries the count it waits for, the entry of the
 // next task and the index of the one after are fetched while this task's dependency is polled
 // (a CTA still works its claims off in table order, which is all that the waits need), and the
-// walk ends when the last grid has converged. @FIG2@
+// walk ends when the last grid has converged: 64 grids 3235 → 2364 µs.
 __global__ void __launch_bounds__(256, 4) batch_kernel(BatchArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int4 s_tk[2];  // the current and the next task (x < 0: none)
