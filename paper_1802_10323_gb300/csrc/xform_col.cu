@@ -2,7 +2,7 @@
 //
 // Same mathematics as the other line transforms (one M-point complex FFT per
 // line of n = 2M reals, with the Table 2 pre/post processing per BC), laid out
-// for lines that are strided in memory. A CTA owns CW = 16 consecutive x columns
+// for lines that are strided in memory. A CTA owns CW (16, or 8) consecutive x columns
 // of one z plane: lane c of each half-warp is column x0 + c, and the TPL threads
 // that share a column split its line, E = M/TPL complex points each.
 //   * Every global access is a row segment of CW consecutive x values (64 bytes
@@ -22,9 +22,10 @@ namespace ps {
 namespace col {
 
 template <class T, int M, bool FWD, int CW>
-__global__ void __launch_bounds__(CShape<M, CW>::NT, sizeof(T) == 4 ? 1024 / CShape<M, CW>::NT : 1)
+__global__ void __launch_bounds__(CShape<T, M, CW>::NT, CShape<T, M, CW>::CTAS)
     xform_col_kernel(FastArgs<T> a) {
-  static_assert(CShape<M, CW>::radix(0) == CShape<M, CW>::E, "the first stage takes all of a thread's points");
+  using S = CShape<T, M, CW>;
+  static_assert(S::radix(0) == S::E, "the first stage takes all of a thread's points");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx<T>* stw = reinterpret_cast<cplx<T>*>(smem_raw);  // ω_M^t, t < M
   cplx<T>* ptw = stw + M;                               // e^{−2πik/n}, k ≤ M
@@ -54,7 +55,7 @@ __global__ void __launch_bounds__(CShape<M, CW>::NT, sizeof(T) == 4 ? 1024 / CSh
 namespace {
 template <class T, int M, bool FWD, int CW>
 cudaError_t launch_col_cw(FastArgs<T> a, cudaStream_t st) {
-  using S = col::CShape<M, CW>;
+  using S = col::CShape<T, M, CW>;
   auto k = col::xform_col_kernel<T, M, FWD, CW>;
   const size_t smem = col::col_smem<T, M, CW>(a.bc);
   static int smem_set = 0;
@@ -81,10 +82,11 @@ cudaError_t launch_col_cw(FastArgs<T> a, cudaStream_t st) {
 }
 }  // namespace
 
-// Tiles of 16 columns: 64-byte rows in FP32, 128-byte rows in FP64.
+// Tiles of 16 columns: 64-byte rows in FP32, 128-byte rows in FP64
 template <class T, int M, bool FWD>
 cudaError_t launch_xform_col(FastArgs<T> a, cudaStream_t st) {
-  constexpr int CW = 16;  // (measured at 1024^3: 8 and 32 columns are slower)
+  // (FP32 1024³: 8 and 32 columns are slower). FP64, M = 256: 8 columns, so that three CTAs fit
+  constexpr int CW = sizeof(T) == 8 && M == 256 ? 8 : 16;
   if (a.axis != 1 || a.ny != 2 * M || a.nx % CW != 0 || a.accumulate || a.amax)
     return cudaErrorInvalidValue;
   return launch_col_cw<T, M, FWD, CW>(a, st);

@@ -137,7 +137,7 @@ __device__ __forceinline__ void gen_stage(const cplx<T>* src, cplx<T>* dst, int 
     if constexpr (R == 3) dft3(v);
     else if constexpr (R == 6) dft6(v);
     else if constexpr (R == 9) dft9(v);
-    else col::dft<T, R, false>(v);
+    else fast::dftR<T, R, false>(v);
     cplx<T>* d = dst + (q * ns * R + k) * ls + l;
 #pragma unroll
     for (int r = 0; r < R; ++r) d[r * ns * ls] = v[r];

@@ -113,7 +113,7 @@ __device__ __forceinline__ void fft_line(cplx<T> (&v)[16], cplx<T>* buf, const L
         v[q * R + r] = cmul(v[q * R + r], w);
       }
     }
-    col::dft<T, R, INV>(&v[q * R]);
+    fast::dftR<T, R, INV>(&v[q * R]);
   }
   if constexpr (STAGE + 1 < S::NST) {
     constexpr int R2 = S::radix(STAGE + 1);

@@ -60,7 +60,7 @@ __device__ __forceinline__ void dft(cplx<T>* v) {
   else if constexpr (R == 9) dft9(v);
   else if constexpr (R == 12) dft12(v);
   else if constexpr (R == 18) dft18(v);
-  else col::dft<T, R, false>(v);
+  else fast::dftR<T, R, false>(v);
 }
 
 // Lines, threads and radices per half length. Threads: the butterflies of a stage in whole

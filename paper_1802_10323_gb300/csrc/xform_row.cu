@@ -24,9 +24,9 @@ namespace ps {
 namespace row {
 
 template <class T, class TI, class TO, int M, bool FWD, int OM>
-__global__ void __launch_bounds__(32 * WARPS, sizeof(T) == 4 ? (M >= 512 ? 3 : 4) : 2)
+__global__ void __launch_bounds__(32 * kWarps<T>, sizeof(T) == 4 ? (M >= 512 ? 3 : 4) : 3)
     xform_row_kernel(FastArgs<T> a) {
-  constexpr int LPW = 32 / Shape<M>::TPL;
+  constexpr int LPW = 32 / Shape<M, kWide<T>>::TPL;
   constexpr int LB = M + M / 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx<T>* stw = reinterpret_cast<cplx<T>*>(smem_raw);
@@ -41,8 +41,8 @@ __global__ void __launch_bounds__(32 * WARPS, sizeof(T) == 4 ? (M >= 512 ? 3 : 4
   // max |transform output| of FP64 outputs, tracked on the values before widening
   // (exact) so that no 64-bit work per value reaches the FP64 pipe
   T tmax = (T)0;
-  const int wstride = gridDim.x * WARPS * LPW;
-  for (int l0 = (blockIdx.x * WARPS + warp) * LPW; l0 < a.nlines; l0 += wstride)
+  const int wstride = gridDim.x * kWarps<T> * LPW;
+  for (int l0 = (blockIdx.x * kWarps<T> + warp) * LPW; l0 < a.nlines; l0 += wstride)
     row_line<T, TI, TO, M, FWD, OM>(a, stw, ptw, xtw, bufs + warp * LPW * LB, l0, tmax);
   if constexpr (sizeof(TO) == 8) {
     if (a.amax) {
@@ -59,33 +59,33 @@ __global__ void __launch_bounds__(32 * WARPS, sizeof(T) == 4 ? (M >= 512 ? 3 : 4
 namespace {
 template <class T, class TI, class TO, int M, bool FWD, int OM>
 cudaError_t launch_row_mode(FastArgs<T> a, cudaStream_t st) {
-  using S = fast::Shape<M>;
+  using S = fast::Shape<M, row::kWide<T>>;
   constexpr int LPW = 32 / S::TPL;
   constexpr size_t LB = M + M / 8;
   auto k = row::xform_row_kernel<T, TI, TO, M, FWD, OM>;
-  const size_t smem = fast_table_bytes<T, M>(a.bc) + (size_t)row::WARPS * LPW * LB * sizeof(cplx<T>);
+  const size_t smem = fast_table_bytes<T, M>(a.bc) + (size_t)row::kWarps<T> * LPW * LB * sizeof(cplx<T>);
   static int smem_set = 0;
   static int blocks_per_sm[2] = {};
   if (!smem_set) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(fast_table_bytes<T, M>(1) + row::WARPS * LPW * LB * sizeof(cplx<T>)));
+                                         (int)(fast_table_bytes<T, M>(1) + row::kWarps<T> * LPW * LB * sizeof(cplx<T>)));
     if (e != cudaSuccess) return e;
     smem_set = 1;
   }
   int& bps = blocks_per_sm[a.bc != 0];
   if (bps == 0) {
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k, 32 * row::WARPS, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k, 32 * row::kWarps<T>, smem);
     if (e != cudaSuccess) return e;
     if (bps < 1) bps = 1;
   }
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int per_cta = row::WARPS * LPW;
+  const int per_cta = row::kWarps<T> * LPW;
   const int ctas = (a.nlines + per_cta - 1) / per_cta;
   const int grid = ctas < sms * bps ? ctas : sms * bps;
   (void)cudaGetLastError();  // a stale error from elsewhere must not be blamed here
-  return launch_k(k, grid, 32 * row::WARPS, smem, st, a);
+  return launch_k(k, grid, 32 * row::kWarps<T>, smem, st, a);
 }
 }  // namespace
 

@@ -18,8 +18,8 @@ namespace ps {
 // anyway (or in a fused multiply-add with the split's sum, split_scale): the results
 // keep their bits, and the FP64 passes, which the FP64 pipe bounds, lose a quarter of
 // their arithmetic outside the FFT stages (NN pair of wavenumbers, forward 32 → 20
-// instructions, backward 36 → 20). FP64 256³ (DD, ND, NN) 2945 → 2647 µs; FP32 passes
-// are bound by memory and keep their time.
+// instructions, backward 36 → 20). FP64 256³ (DD, ND, NN) 2945 → 2647 µs; FP32
+// passes are bound by memory and keep their time.
 template <class T, int M, bool FWD>
 __device__ __forceinline__ void load_line_tables(const cplx<T>* tw, int bc, cplx<T>* stw) {
   constexpr int N = 2 * M;
@@ -67,7 +67,12 @@ struct alignas(sizeof(T) * N) vec {
   T v[N];
 };
 
-constexpr int WARPS = 8;  // warps per CTA
+// Warps per CTA and wide stages (fast::Shape) for FP64: few warps with many registers, the
+// pipe needs no more
+template <class T>
+constexpr int kWarps = sizeof(T) == 8 ? 4 : 8;
+template <class T>
+constexpr bool kWide = sizeof(T) == 8;
 
 template <class TC, class TI>
 __device__ __forceinline__ TC in_cvt(TI x) { return ld_cvt<TC, TI>::f(x); }
@@ -102,11 +107,13 @@ struct LaneSlots {
 
 // One line (two for M = 64, half a warp each) of the x transform: the warp's
 // exchange buffers at bufs, tables in shared memory, the first line index l0.
-// tmax accumulates max |FP64 output| (before widening; an FP64 transform only when asked, on its own pipe) for the caller's reduction.
+// tmax accumulates max |FP64 output| for the caller's reduction (before widening; FP64
+// transforms only when asked: the comparison costs their pipe).
 template <class T, class TI, class TO, int M, bool FWD, int OM>
 __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* stw, const cplx<T>* ptw,
                                          const cplx<T>* xtw, cplx<T>* bufs, int l0, T& tmax) {
-  using S = Shape<M>;
+  constexpr bool W = kWide<T>;
+  using S = Shape<M, W>;
   constexpr int N = 2 * M, E = S::E, TPL = S::TPL;
   constexpr int R0 = S::radix(0), RL = S::radix(S::NST - 1);
   constexpr int LB = M + M / 8;  // complex slots of a line's exchange buffer (skewed)
@@ -188,7 +195,7 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
 #pragma unroll
       for (int si = 0; si < E; ++si) v[si] = cscale(v[si], s);
     }
-    fast::fft_stages<T, M, false, 0, 1>(v, lc, stw, t);
+    fast::fft_stages<T, M, false, 0, 1, W>(v, lc, stw, t);
     if constexpr (TPL == 32) {
       // ---- post-processing in registers: pairs (k, M−k), Z_{M−k} from the partner lane ----
       // Lane t takes its slots j < E/2 (k = t + 32j) and writes the outputs of k and of
@@ -213,11 +220,17 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
         const bool rev = (bc == BC_DD);
         auto OUTQ = [&](int q, T val) { Y(rev ? (N - 1 - q) : q, val); };
         // outputs of k (and of M − k unless k = 0 or 2k = M) from Z_k and Z_{M−k}
-        auto pair_out = [&](int k, cplx<T> Zk, cplx<T> Zmk) {
-          const cplx<T> Ek = cadd(Zk, conj_(Zmk));
-          const cplx<T> Ok = mul_mi(csub(Zk, conj_(Zmk)));
-          const cplx<T> B = cmul(ptw[k], Ok);
-          const cplx<T> Vk = split_add(Ek, B, h), Vmk = conj_(split_sub(Ek, B, h));
+        auto pair_out = [&](int k, cplx<T> Zk, cplx<T> Zmk, bool self) {
+          cplx<T> Vk, Vmk;
+          if (self) {  // k = M/2 is its own partner
+            Vk = Vmk = cscale(conj_(Zk), (T)2 * h);
+          } else {
+            const cplx<T> Ek = cadd(Zk, conj_(Zmk));
+            const cplx<T> Ok = mul_mi(csub(Zk, conj_(Zmk)));
+            const cplx<T> B = cmul(ptw[k], Ok);
+            Vk = split_add(Ek, B, h);
+            Vmk = conj_(split_sub(Ek, B, h));
+          }
           if (bc == BC_P) {
             if (k == 0) {
               Y(0, Vk.x);
@@ -252,9 +265,9 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
                                 __shfl_sync(full, v[LS::sout(E - 1 - j)].y, pl)};
           const cplx<T> Zmk = (t != 0) ? recv : (j == 0 ? Zk : prev);
           prev = recv;
-          pair_out(t + 32 * j, Zk, Zmk);
+          pair_out(t + 32 * j, Zk, Zmk, false);
         }
-        if (t == 0) pair_out(M / 2, prev, prev);  // k = M/2 pairs with itself
+        if (t == 0) pair_out(M / 2, prev, prev, true);
       }
     } else {
       // ---- post-processing: pairs (k, M−k) through the exchange buffer, scalar stores ----
@@ -282,10 +295,16 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
           const int k = t + i * TPL;
           if (k > M / 2) break;
           const cplx<T> Zk = lc[cpad(k)], Zmk = lc[cpad(k == 0 ? 0 : M - k)];
-          const cplx<T> Ek = cadd(Zk, conj_(Zmk));
-          const cplx<T> Ok = mul_mi(csub(Zk, conj_(Zmk)));
-          const cplx<T> B = cmul(ptw[k], Ok);
-          const cplx<T> Vk = split_add(Ek, B, h), Vmk = conj_(split_sub(Ek, B, h));
+          cplx<T> Vk, Vmk;
+          if (i == NP - 1) {  // k = M/2 is its own partner
+            Vk = Vmk = cscale(conj_(Zk), (T)2 * h);
+          } else {
+            const cplx<T> Ek = cadd(Zk, conj_(Zmk));
+            const cplx<T> Ok = mul_mi(csub(Zk, conj_(Zmk)));
+            const cplx<T> B = cmul(ptw[k], Ok);
+            Vk = split_add(Ek, B, h);
+            Vmk = conj_(split_sub(Ek, B, h));
+          }
           if (bc == BC_P) {
             if (k == 0) {
               Y(0, Vk.x);
@@ -405,55 +424,53 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
           lc[cpad(k)] = cmul(v[i], xtw[k]);
         }
       } else {
-        constexpr int NP = (M / 2) / TPL + 1;
-        T xv[NP][4];
-  #pragma unroll
+        constexpr int NP = (M / 2) / TPL;  // pairs (k, M − k) of a thread; k = M/2, its own partner, is t = 0's
+        const bool rev = (bc == BC_DD);
+        T xv[NP][4], xs[2] = {(T)0, (T)0};
+#pragma unroll
         for (int i = 0; i < NP; ++i) {
           const int k = t + i * TPL;
-          const bool ok = (i < NP - 1) || (k <= M / 2);
           int q[4];
-          bool use[4] = {ok, ok, ok, ok};
+          bool use[4] = {true, true, true, true};
           if (bc == BC_P) {
             q[0] = k == 0 ? 0 : 2 * k - 1;
             q[1] = 2 * k;
             q[2] = k == 0 ? N - 1 : 2 * (M - k) - 1;
             q[3] = 2 * (M - k);
-            use[1] = use[3] = ok && k != 0;
+            use[1] = use[3] = k != 0;
           } else {
-            const bool rev = (bc == BC_DD);
             const int qq[4] = {k, N - k, M - k, N - M + k};
-  #pragma unroll
+#pragma unroll
             for (int u = 0; u < 4; ++u) {
               q[u] = rev ? (N - 1 - qq[u]) : qq[u];
-              use[u] = ok && qq[u] < N;
+              use[u] = qq[u] < N;
             }
           }
-  #pragma unroll
+#pragma unroll
           for (int u = 0; u < 4; ++u) xv[i][u] = use[u] ? X(q[u]) : (T)0;
         }
-  #pragma unroll
+        if (t == 0) {
+          xs[0] = X(bc == BC_P ? M - 1 : (rev ? N - 1 - M / 2 : M / 2));
+          xs[1] = X(bc == BC_P ? M : (rev ? M / 2 - 1 : N - M / 2));
+        }
+        auto V = [&](int k, T x0, T x1) {
+          if (bc == BC_P) return cplx<T>{x0, -x1};
+          cplx<T> w = xtw[k];
+          w.y = -w.y;
+          return cmul(w, cplx<T>{x0, -x1});
+        };
+#pragma unroll
         for (int i = 0; i < NP; ++i) {
           const int k = t + i * TPL;
-          if (i == NP - 1 && k > M / 2) break;
-          cplx<T> Vk, Vm;
-          if (bc == BC_P) {
-            Vk = {xv[i][0], -xv[i][1]};
-            Vm = {xv[i][2], -xv[i][3]};
-          } else {
-            cplx<T> w = xtw[k];
-            w.y = -w.y;
-            Vk = cmul(w, cplx<T>{xv[i][0], -xv[i][1]});
-            cplx<T> w2 = xtw[M - k];
-            w2.y = -w2.y;
-            Vm = cmul(w2, cplx<T>{xv[i][2], -xv[i][3]});
-          }
+          const cplx<T> Vk = V(k, xv[i][0], xv[i][1]), Vm = V(M - k, xv[i][2], xv[i][3]);
           const cplx<T> Ek = cadd(Vk, conj_(Vm));
           cplx<T> wn = ptw[k];
           wn.y = -wn.y;
           const cplx<T> Ok = cmul(csub(Vk, conj_(Vm)), wn);
-          if (k < M) lc[cpad(k)] = split_add(Ek, mul_i(Ok), h);
-          if (k != 0 && 2 * k != M) lc[cpad(M - k)] = split_add(conj_(Ek), mul_i(conj_(Ok)), h);
+          lc[cpad(k)] = split_add(Ek, mul_i(Ok), h);
+          if (k != 0) lc[cpad(M - k)] = split_add(conj_(Ek), mul_i(conj_(Ok)), h);
         }
+        if (t == 0) lc[cpad(M / 2)] = cscale(conj_(V(M / 2, xs[0], xs[1])), (T)2 * h);
       }
       __syncwarp();
   #pragma unroll
@@ -461,8 +478,8 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
   #pragma unroll
         for (int r = 0; r < R0; ++r) v[q * R0 + r] = lc[cpad(t + q * TPL + r * (M / R0))];
     }
-    if (bc_iv(bc)) fast::fft_stages<T, M, false, 0, 1>(v, lc, stw, t);
-    else fast::fft_stages<T, M, true, 0, 1>(v, lc, stw, t);
+    if (bc_iv(bc)) fast::fft_stages<T, M, false, 0, 1, W>(v, lc, stw, t);
+    else fast::fft_stages<T, M, true, 0, 1, W>(v, lc, stw, t);
     __syncwarp();  // the last stage's buffer reads are done before the next line
     // ---- backward outputs straight from the last stage, as vectors ----
     // slot si = q·RL + r holds wavenumber k = t + q·TPL + r·(M/RL); k < M/2 iff r < RL/2
@@ -548,70 +565,32 @@ __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* st
 
 namespace col {
 
-template <int M, int CW>  // CW: x columns per CTA (16 or 8)
+template <class T, int M, int CW>  // CW: x columns per CTA
 struct CShape {
-  static constexpr int TPL = (M >= 128) ? 32 : 16;  // threads per column
+  static constexpr bool W = sizeof(T) == 8;  // FP64: the wide stages of fast::Shape
+  static constexpr int TPL = W ? fast::Shape<M, true>::TPL : (M >= 128) ? 32 : 16;  // threads per column
   static constexpr int E = M / TPL;                 // complex points per thread
   static constexpr int NT = CW * TPL;               // threads per CTA
-  static constexpr int NST = (M == 128) ? 4 : 3;
-  // radix of stage s; the first equals E (one butterfly per thread), all divide E
+  // resident CTAs: FP64 keeps 168 registers a thread (three CTAs of 128), FP32 64
+  static constexpr int CTAS = !W ? 1024 / NT : (NT <= 384 ? 384 / NT : 1);
+  static constexpr int NST = W ? fast::Shape<M, true>::NST : (M == 128) ? 4 : 3;
+  // radix of stage s, a divisor of E
   __host__ __device__ static constexpr int radix(int s) {
-    return (M == 512) ? (s == 0 ? 16 : (s == 1 ? 8 : 4))
-         : (M == 256) ? (s < 2 ? 8 : 4)
+    if (M == 512) return s == 0 ? 16 : (s == 1 ? 8 : 4);
+    if (W) return fast::Shape<M, true>::radix(s);
+    return (M == 256) ? (s < 2 ? 8 : 4)
          : (M == 128) ? (s < 3 ? 4 : 2)
          : 4;
   }
 };
 
-// 16-point DFT in natural order, as 4 × 4: X[k1 + 4k2] =
-// Σ_{n2} W4^{n2·k2} · W16^{n2·k1} · Σ_{n1} x[n2 + 4n1] · W4^{n1·k1}.
-template <class T, bool INV>
-__device__ __forceinline__ void dft16(cplx<T>* v) {
-  const T c1 = (T)0.92387953251128675613, s1 = (T)0.38268343236508977173;  // cos, sin of π/8
-  const T h = (T)0.70710678118654752440;
-  cplx<T> a[4][4];
-#pragma unroll
-  for (int n2 = 0; n2 < 4; ++n2) {
-#pragma unroll
-    for (int n1 = 0; n1 < 4; ++n1) a[n2][n1] = v[n2 + 4 * n1];
-    fast::dft4<T, INV>(a[n2]);
-  }
-  // W16^m = (cos 2πm/16, −sin 2πm/16) for the forward transform, conjugate for the inverse
-  auto tw = [&](cplx<T> z, T wr, T wi) {
-    if (INV) wi = -wi;
-    return cplx<T>{z.x * wr - z.y * wi, z.x * wi + z.y * wr};
-  };
-  a[1][1] = tw(a[1][1], c1, -s1);  // m = 1
-  a[1][2] = tw(a[1][2], h, -h);    // m = 2
-  a[1][3] = tw(a[1][3], s1, -c1);  // m = 3
-  a[2][1] = tw(a[2][1], h, -h);    // m = 2
-  a[2][2] = INV ? mul_i(a[2][2]) : mul_mi(a[2][2]);  // m = 4
-  a[2][3] = tw(a[2][3], -h, -h);   // m = 6
-  a[3][1] = tw(a[3][1], s1, -c1);  // m = 3
-  a[3][2] = tw(a[3][2], -h, -h);   // m = 6
-  a[3][3] = tw(a[3][3], -c1, s1);  // m = 9
-#pragma unroll
-  for (int k1 = 0; k1 < 4; ++k1) {
-    cplx<T> b[4] = {a[0][k1], a[1][k1], a[2][k1], a[3][k1]};
-    fast::dft4<T, INV>(b);
-#pragma unroll
-    for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = b[k2];
-  }
-}
-
-template <class T, int R, bool INV>
-__device__ __forceinline__ void dft(cplx<T>* v) {
-  if constexpr (R == 16) dft16<T, INV>(v);
-  else fast::dftR<T, R, INV>(v);
-}
-
 // Stages STAGE… of the M-point FFT of this thread's column. On entry
 // v[q·R + r] = x[b_q + r·M/R] with b_q = b + q·TPL; on return v holds the last
 // stage's outputs, v[q·R + r] at position b_q + r·(M/R_last).
 template <class T, int M, int CW, bool INV, int STAGE, int NS>
-__device__ __forceinline__ void fft_col(cplx<T> (&v)[CShape<M, CW>::E], cplx<T>* buf, const cplx<T>* stw,
+__device__ __forceinline__ void fft_col(cplx<T> (&v)[CShape<T, M, CW>::E], cplx<T>* buf, const cplx<T>* stw,
                                         int b, int c) {
-  using S = CShape<M, CW>;
+  using S = CShape<T, M, CW>;
   constexpr int E = S::E, TPL = S::TPL;
   constexpr int R = S::radix(STAGE);
 #pragma unroll
@@ -626,7 +605,7 @@ __device__ __forceinline__ void fft_col(cplx<T> (&v)[CShape<M, CW>::E], cplx<T>*
         v[q * R + r] = cmul(v[q * R + r], w);
       }
     }
-    dft<T, R, INV>(&v[q * R]);
+    fast::dftR<T, R, INV>(&v[q * R]);
   }
   if constexpr (STAGE + 1 < S::NST) {
     constexpr int R2 = S::radix(STAGE + 1);
@@ -660,7 +639,7 @@ __host__ __device__ constexpr size_t col_smem(int bc) {
 template <class T, int M, bool FWD, int CW>
 __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* stw, const cplx<T>* ptw,
                                          const cplx<T>* xtw, cplx<T>* buf, int g) {
-  using S = CShape<M, CW>;
+  using S = CShape<T, M, CW>;
   constexpr int N = 2 * M, E = S::E, TPL = S::TPL;
   constexpr int RL = S::radix(S::NST - 1);
   const int bc = a.bc;
@@ -734,10 +713,16 @@ __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* st
         const int k = b + i * TPL;
         if (k > M / 2) break;
         const cplx<T> Zk = buf[k * CW + c], Zmk = buf[(k == 0 ? 0 : M - k) * CW + c];
-        const cplx<T> Ek = cadd(Zk, conj_(Zmk));
-        const cplx<T> Ok = mul_mi(csub(Zk, conj_(Zmk)));
-        const cplx<T> B = cmul(ptw[k], Ok);
-        const cplx<T> Vk = split_add(Ek, B, h), Vmk = conj_(split_sub(Ek, B, h));
+        cplx<T> Vk, Vmk;
+        if (i == NP - 1) {  // k = M/2 is its own partner
+          Vk = Vmk = cscale(conj_(Zk), (T)2 * h);
+        } else {
+          const cplx<T> Ek = cadd(Zk, conj_(Zmk));
+          const cplx<T> Ok = mul_mi(csub(Zk, conj_(Zmk)));
+          const cplx<T> B = cmul(ptw[k], Ok);
+          Vk = split_add(Ek, B, h);
+          Vmk = conj_(split_sub(Ek, B, h));
+        }
         if (bc == BC_P) {
           if (k == 0) {
             Y(0, Vk.x);
@@ -779,55 +764,53 @@ __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* st
       }
     } else {
       // all row loads of the pairs first (they are independent), then the arithmetic
-      constexpr int NP = (M / 2) / TPL + 1;  // pairs per thread; only b = 0 has k = M/2 in the last
-      T xv[NP][4];
+      constexpr int NP = (M / 2) / TPL;  // pairs (k, M − k) of a thread; k = M/2, its own partner, is b = 0's
+      const bool rev = (bc == BC_DD);
+      T xv[NP][4], xs[2] = {(T)0, (T)0};
 #pragma unroll
       for (int i = 0; i < NP; ++i) {
         const int k = b + i * TPL;
-        const bool ok = (i < NP - 1) || (k <= M / 2);
         int q[4];
-        bool use[4] = {ok, ok, ok, ok};
+        bool use[4] = {true, true, true, true};
         if (bc == BC_P) {
           q[0] = k == 0 ? 0 : 2 * k - 1;
           q[1] = 2 * k;
           q[2] = k == 0 ? N - 1 : 2 * (M - k) - 1;
           q[3] = 2 * (M - k);
-          use[1] = use[3] = ok && k != 0;
+          use[1] = use[3] = k != 0;
         } else {
-          const bool rev = (bc == BC_DD);
           const int qq[4] = {k, N - k, M - k, N - M + k};
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
             q[u] = rev ? (N - 1 - qq[u]) : qq[u];
-            use[u] = ok && qq[u] < N;
+            use[u] = qq[u] < N;
           }
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) xv[i][u] = use[u] ? X(q[u]) : (T)0;
       }
+      if (b == 0) {
+        xs[0] = X(bc == BC_P ? M - 1 : (rev ? N - 1 - M / 2 : M / 2));
+        xs[1] = X(bc == BC_P ? M : (rev ? M / 2 - 1 : N - M / 2));
+      }
+      auto V = [&](int k, T x0, T x1) {
+        if (bc == BC_P) return cplx<T>{x0, -x1};
+        cplx<T> w = xtw[k];
+        w.y = -w.y;
+        return cmul(w, cplx<T>{x0, -x1});
+      };
 #pragma unroll
       for (int i = 0; i < NP; ++i) {
         const int k = b + i * TPL;
-        if (i == NP - 1 && k > M / 2) break;
-        cplx<T> Vk, Vm;
-        if (bc == BC_P) {
-          Vk = {xv[i][0], -xv[i][1]};
-          Vm = {xv[i][2], -xv[i][3]};
-        } else {
-          cplx<T> w = xtw[k];
-          w.y = -w.y;
-          Vk = cmul(w, cplx<T>{xv[i][0], -xv[i][1]});
-          cplx<T> w2 = xtw[M - k];
-          w2.y = -w2.y;
-          Vm = cmul(w2, cplx<T>{xv[i][2], -xv[i][3]});
-        }
+        const cplx<T> Vk = V(k, xv[i][0], xv[i][1]), Vm = V(M - k, xv[i][2], xv[i][3]);
         const cplx<T> Ek = cadd(Vk, conj_(Vm));
         cplx<T> wn = ptw[k];
         wn.y = -wn.y;
         const cplx<T> Ok = cmul(csub(Vk, conj_(Vm)), wn);
-        if (k < M) buf[k * CW + c] = split_add(Ek, mul_i(Ok), h);
-        if (k != 0 && 2 * k != M) buf[(M - k) * CW + c] = split_add(conj_(Ek), mul_i(conj_(Ok)), h);
+        buf[k * CW + c] = split_add(Ek, mul_i(Ok), h);
+        if (k != 0) buf[(M - k) * CW + c] = split_add(conj_(Ek), mul_i(conj_(Ok)), h);
       }
+      if (b == 0) buf[(M / 2) * CW + c] = cscale(conj_(V(M / 2, xs[0], xs[1])), (T)2 * h);
     }
     __syncthreads();
 #pragma unroll
