@@ -981,15 +981,25 @@ cudaError_t launch_residual_exact(const ResidArgs& a, cudaStream_t st) {
 
 namespace {
 // Σ over the per-block partials of (Δz^f·r, Δz^f·f) in double-float, one CTA;
-// thread 0 gets them in FP64.
+// the threads of its first warp get them in FP64. A chain of latencies: four loads are in
+// flight a thread, and the warps' sums are added in a tree (an FP64 addition takes 33 ns).
+// The finalize kernel: 22.7 → 7.6 µs at 1024³, 13.7 → 7.6 at 384×288×201, 10.5 → 6.1 at 128³.
 __device__ void sum_partials(const float* partial, int nblocks, double& sr_out, double& sf_out) {
   __shared__ df sr[32], sf[32];
   df ar = {0.f, 0.f}, af = {0.f, 0.f};
   const float4* pv = reinterpret_cast<const float4*>(partial);
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-    const float4 v = pv[b];
-    ar = add_u(ar, df{v.x, v.y});
-    af = add_u(af, df{v.z, v.w});
+  for (int b = threadIdx.x; b < nblocks; b += 4 * blockDim.x) {
+    float4 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int bq = b + q * (int)blockDim.x;
+      v[q] = bq < nblocks ? pv[bq] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      ar = add_u(ar, df{v[q].x, v[q].y});
+      af = add_u(af, df{v[q].z, v[q].w});
+    }
   }
   for (int o = 16; o > 0; o >>= 1) {
     ar = add_u(ar, df{__shfl_xor_sync(0xffffffffu, ar.h, o), __shfl_xor_sync(0xffffffffu, ar.l, o)});
@@ -1001,11 +1011,16 @@ __device__ void sum_partials(const float* partial, int nblocks, double& sr_out, 
   }
   __syncthreads();
   double s1 = 0.0, s2 = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      s1 += (double)sr[w].h + (double)sr[w].l;
-      s2 += (double)sf[w].h + (double)sf[w].l;
+  if (threadIdx.x < 32) {
+    if (threadIdx.x < (blockDim.x >> 5)) {
+      s1 = (double)sr[threadIdx.x].h + (double)sr[threadIdx.x].l;
+      s2 = (double)sf[threadIdx.x].h + (double)sf[threadIdx.x].l;
     }
+    for (int o = 16; o > 0; o >>= 1) {
+      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+    }
+  }
   sr_out = s1;
   sf_out = s2;
 }
@@ -1032,7 +1047,8 @@ __global__ void __launch_bounds__(1024) finalize_kernel(Ctrl* c, const float* pa
                                                         int iteration, int attempt, int last,
                                                         double anorm, const int* skip, ps_info* info) {
   pdl_wait();
-  if ((skip && *skip) || c->converged) return;
+  const Ctrl in = *c;  // read once, under the latency of the partials
+  if ((skip && *skip) || in.converged) return;
   double s1 = 0.0, s2 = 0.0;
   if (singular) sum_partials(partial, nblocks, s1, s2);
   if (threadIdx.x != 0) return;
@@ -1046,20 +1062,20 @@ __global__ void __launch_bounds__(1024) finalize_kernel(Ctrl* c, const float* pa
       c->mu[0] = h;
       c->mu[1] = (float)(mf - (double)h);
     } else {
-      mf = c->mf;
+      mf = in.mf;
     }
   }
-  if (iteration > 0)
-    c->bnd += anorm * (ldexp(bits_f64(c->dmax), -39) + ldexp(bits_f64(c->pmax), -52));
-  c->dmax_prev = c->dmax;  // the scale of the output repeat of this pass
+  double bnd = in.bnd;
+  if (iteration > 0) c->bnd = bnd += anorm * (ldexp(bits_f64(in.dmax), -39) + ldexp(bits_f64(in.pmax), -52));
+  c->dmax_prev = in.dmax;  // the scale of the output repeat of this pass
   c->dmax = 0;             // the next correction's x backward records max|e| here
-  const double rmax = red_max_value(c->red[0]), rmin = red_min_value(c->red[1]);
-  const double vfmax = red_max_value(c->red[2]), vfmin = red_min_value(c->red[3]);
+  const double rmax = red_max_value(in.red[0]), rmin = red_min_value(in.red[1]);
+  const double vfmax = red_max_value(in.red[2]), vfmin = red_min_value(in.red[3]);
   const double rn = fmax(rmax - mr, mr - rmin);
   const double fn = fmax(vfmax - mf, mf - vfmin);
   const double rel = fn > 0 ? rn / fn : (rn > 0 ? INFINITY : 0.0);
   if (iteration == 0 && attempt == 0) {
-    const bool redo = ldexp(anorm * bits_f64(c->pmax), -43) > 0.05 * rtol * fn;
+    const bool redo = ldexp(anorm * bits_f64(in.pmax), -43) > 0.05 * rtol * fn;
     c->skip_redo = redo ? 0 : 1;
     c->nomat0 = 1;
     if (redo) {  // the repeated pass reduces f again
@@ -1074,7 +1090,7 @@ __global__ void __launch_bounds__(1024) finalize_kernel(Ctrl* c, const float* pa
   c->iterations = iteration;
   const bool ok = rel <= rtol;
   if (ok) c->converged = 1;
-  if (ok || last) c->vskip = (c->bnd <= 0.05 * rtol * fn) ? 1 : 0;
+  if (ok || last) c->vskip = (bnd <= 0.05 * rtol * fn) ? 1 : 0;
   if (iteration == 0) c->nomat0 = (ok || last) ? 0 : 1;
   c->skip_out = (ok || last) ? 1 : 0;
   if (info && (ok || last)) {
@@ -1117,13 +1133,13 @@ __global__ void __launch_bounds__(1024) finalize_exact_kernel(Ctrl* c, const flo
 cudaError_t launch_finalize(Ctrl* ctrl, const float* partial, int nblocks, double wsum_total,
                             int singular, double rtol, int iteration, int attempt, int last,
                             double anorm, const int* skip, ps_info* info, cudaStream_t st) {
-  return launch_k(finalize_kernel, 1, 1024, 0, st, ctrl, partial, nblocks, wsum_total, singular, rtol, iteration,
+  return launch_k(finalize_kernel, 1, singular ? 1024 : 32, 0, st, ctrl, partial, nblocks, wsum_total, singular, rtol, iteration,
                   attempt, last, anorm, skip, info);
 }
 
 cudaError_t launch_finalize_exact(Ctrl* ctrl, const float* partial, int nblocks, double wsum_total,
                                   int singular, double rtol, ps_info* info, cudaStream_t st) {
-  return launch_k(finalize_exact_kernel, 1, 1024, 0, st, ctrl, partial, nblocks, wsum_total, singular, rtol, info);
+  return launch_k(finalize_exact_kernel, 1, singular ? 1024 : 32, 0, st, ctrl, partial, nblocks, wsum_total, singular, rtol, info);
 }
 
 __global__ void widen_kernel(const float* __restrict__ u, double* __restrict__ p, size_t n, const int* skip) {
