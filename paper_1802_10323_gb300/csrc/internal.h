@@ -95,7 +95,7 @@ template <class T>
 struct ZArgs {
   T* data;                  // [nz][ny][nx], spectral in x and y; overwritten with Φ̂
   T* scr_c;                 // scratch, nx*ny*nz (eliminated upper diagonal)
-  T* scr_u;                 // scratch for the periodic (Sherman–Morrison) column, or null
+  T* scr_u;                 // scratch of a periodic z (carried coefficients), or null
   int nx, ny, nz;
   const T* lamx;            // λ_qx/Δx², nx
   const T* lamy;            // λ_qy/Δy², ny

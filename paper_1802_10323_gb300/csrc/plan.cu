@@ -418,7 +418,7 @@ ZArgs<T> zargs(const ps_plan* p, T* data, void* ws, const WsLayout& L, const int
 
 // The same z systems on planes stored transposed ([n_x][n_y], y fastest), as the
 // long y lines leave them: the column index runs over q_y first, so the x and y
-// roles (lengths, eigenvalues, the FP64 low-wavenumber rectangle) swap. The
+// roles (lengths, eigenvalues, the low-wavenumber rectangle) swap. The
 // elimination scratch is `scratch` (an idle array of n_x·n_y·n_z values of T)
 // instead of the workspace array that now holds the data.
 template <class T>
@@ -1049,25 +1049,33 @@ ps_status ps_plan_create_helmholtz(ps_plan** out, int nx, int ny, int nz, double
   p->dev = dev;
   size_t off = 0;
   {
-    // FP32 paths: columns whose z system has κ ≈ ‖T_z‖/|λ| > 10^5 are solved in
-    // double-float (tridiag.cu; a periodic z needs 32 planes for that). λ grows with q along each axis, so they lie in
-    // the rectangle q_x < lowx, q_y < lowy; at most 1/8 of the columns. A Helmholtz
-    // shift adds α to every |λ| (all terms of the diagonal shift have one sign).
+    // FP32 paths: columns whose z system has κ ≈ ‖T_z‖/|λ| above a limit are solved in
+    // double-float (tridiag.cu; a periodic z needs 32 planes for that). λ grows with q along
+    // each axis, so they lie in the rectangle q_x < lowx, q_y < lowy; at most 1/8 of the
+    // columns. A Helmholtz shift adds α to every |λ| (all terms of the diagonal shift have one
+    // sign). The limit is 10^5, or 10^3 where that makes at most two columns an SM, which run
+    // beside the FP32 columns: on thin or coarse grids the lowest modes carry the solution,
+    // and a column's FP32 error is about ε·κ (4096×4096×16
+    // after one correction: 1.2e-9 with 10^5 alone, 5–6e-10; the z pass keeps its 387 µs).
     p->lowx = p->lowy = 0;
     if (prec != PS_FP64 && (bcz != PS_BC_PERIODIC || nz >= 32)) {
       double zmax = 0.0;
       for (int k = 0; k < nz; ++k)
         zmax = std::max(zmax, std::fabs(za[k]) + std::fabs(zb[k]) + std::fabs(zc[k]));
-      const double thr = zmax / 1e5;
       const std::vector<double> lx = eig_scaled(bcx, nx, dx), ly = eig_scaled(bcy, ny, dy);
-      int qx = 0, qy = 0;
-      while (qx < nx && std::fabs(lx[qx]) + alpha < thr) ++qx;
-      while (qy < ny && std::fabs(ly[qy]) + alpha < thr) ++qy;
-      while ((size_t)qx * qy * 8 > (size_t)nx * ny && qy > 1) --qy;
-      while ((size_t)qx * qy * 8 > (size_t)nx * ny && qx > 1) --qx;
-      if ((size_t)qx * qy * 8 <= (size_t)nx * ny && qx > 0 && qy > 0) {
-        p->lowx = qx;
-        p->lowy = qy;
+      for (const double limit : {1e3, 1e5}) {
+        p->lowx = p->lowy = 0;
+        const double thr = zmax / limit;
+        int qx = 0, qy = 0;
+        while (qx < nx && std::fabs(lx[qx]) + alpha < thr) ++qx;
+        while (qy < ny && std::fabs(ly[qy]) + alpha < thr) ++qy;
+        while ((size_t)qx * qy * 8 > (size_t)nx * ny && qy > 1) --qy;
+        while ((size_t)qx * qy * 8 > (size_t)nx * ny && qx > 1) --qx;
+        if ((size_t)qx * qy * 8 <= (size_t)nx * ny && qx > 0 && qy > 0) {
+          p->lowx = qx;
+          p->lowy = qy;
+        }
+        if (p->lowx * p->lowy <= 304) break;
       }
     }
   }
