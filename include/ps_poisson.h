@@ -82,7 +82,8 @@ typedef enum {
  *   PS_FP32_REFINE  FP64 fields; FP32 bulk transforms and tridiagonal solves,
  *                   iterative refinement whose residual r = f − A·Φ is formed
  *                   in double-float (pairs of FP32) from the FP64 fields, until
- *                   ‖r‖∞ ≤ rtol·‖f_c‖∞ or max_iter corrections. */
+ *                   ‖r‖∞ ≤ rtol·‖f_c‖∞ or max_iter corrections (the first correction
+ *                   ends it at half of rtol while another is allowed). */
 typedef enum { PS_FP64 = 0, PS_FP32 = 1, PS_FP32_REFINE = 2 } ps_precision;
 
 /* Device-side record written by every solve (caller allocates it in device
