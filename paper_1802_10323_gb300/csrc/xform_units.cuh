@@ -643,7 +643,16 @@ __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* st
   constexpr int N = 2 * M, E = S::E, TPL = S::TPL;
   constexpr int RL = S::radix(S::NST - 1);
   const int bc = a.bc;
-  const int c = threadIdx.x % CW, b = threadIdx.x / CW;
+  const int c = threadIdx.x % CW;
+  // PAIR: the half-warps of warp w are b = w and 32 − w (0 and 16 for w = 0), so that the
+  // thread holding wavenumber k = b + 32·j and the one holding M − k = (32 − b) + 32·(E−1−j)
+  // are lanes apart by 16, or the same thread (b = 0: slot E − j; b = 16: slot E − 1 − j): the
+  // pairs of Table 2 meet by shuffle instead of through the buffer (forward and backward,
+  // µs: 512×256×256 78 → 74 and 84 → 81, 512³ 250 → 233 and 296 → 290, 1024³ 1881 → 1835
+  // forward; backward M = 512 holds too many values for it: 2277 → 2322, so it keeps the buffer).
+  constexpr bool PAIR = TPL == 32 && CW == 16 && (FWD || M < 512);
+  const int wi = threadIdx.x / 32, hb = (threadIdx.x / CW) & 1;
+  const int b = !PAIR ? (int)threadIdx.x / CW : (hb == 0 ? wi : (wi == 0 ? 16 : 32 - wi));
   const T* in = static_cast<const T*>(a.in);  // may equal out (in-place y passes)
   T* out = static_cast<T*>(a.out);
   const int nx = a.nx, ny = a.ny;
@@ -691,76 +700,105 @@ __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* st
       for (int r = 0; r < E; ++r) v[r] = cscale(v[r], s);
     }
     fft_col<T, M, CW, false, 0, 1>(v, buf, stw, b, c);
-    // ---- post-processing: pair k with M − k through the buffer, rows out ----
-    __syncthreads();
+    // ---- post-processing: pairs (k, M − k), rows out ----
+    const bool rev = (bc == BC_DD);
+    auto OUTQ = [&](int q, T val) { Y(rev ? (N - 1 - q) : q, val); };
+    auto pair_out = [&](int k, cplx<T> Zk, cplx<T> Zmk, bool self) {
+      cplx<T> Vk, Vmk;
+      if (self) {  // k = M/2 is its own partner
+        Vk = Vmk = cscale(conj_(Zk), (T)2 * h);
+      } else {
+        const cplx<T> Ek = cadd(Zk, conj_(Zmk));
+        const cplx<T> Ok = mul_mi(csub(Zk, conj_(Zmk)));
+        const cplx<T> B = cmul(ptw[k], Ok);
+        Vk = split_add(Ek, B, h);
+        Vmk = conj_(split_sub(Ek, B, h));
+      }
+      if (bc == BC_P) {
+        if (k == 0) {
+          Y(0, Vk.x);
+          Y(N - 1, Vmk.x);
+        } else {
+          Y(2 * k - 1, Vk.x);
+          Y(2 * k, -Vk.y);
+          if (2 * k != M) {
+            Y(2 * (M - k) - 1, Vmk.x);
+            Y(2 * (M - k), -Vmk.y);
+          }
+        }
+      } else {
+        if (k == 0) {
+          OUTQ(0, Vk.x);
+          OUTQ(M, (T)0.70710678118654752440 * Vmk.x);
+        } else {
+          const cplx<T> c1 = cmul(xtw[k], Vk);
+          OUTQ(k, c1.x);
+          OUTQ(N - k, -c1.y);
+          if (2 * k != M) {
+            const cplx<T> c2 = cmul(xtw[M - k], Vmk);
+            OUTQ(M - k, c2.x);
+            OUTQ(M + k, -c2.y);
+          }
+        }
+      }
+    };
+    if constexpr (PAIR) {
+      // slot si holds j = si / RL + (si % RL)·(M/RL/32)
+      auto so = [](int j) { return (j % (E / RL)) * RL + j / (E / RL); };
+      if (bc_iv(bc)) {
 #pragma unroll
-    for (int q = 0; q < E / RL; ++q)
+        for (int j = 0; j < E; ++j) {
+          const int k = b + 32 * j;
+          const cplx<T> cc = cmul(xtw[M + k], v[so(j)]);
+          Y(2 * k, cc.x);
+          Y(N - 1 - 2 * k, -cc.y);
+        }
+      } else {
 #pragma unroll
-      for (int r = 0; r < RL; ++r) buf[(b + q * TPL + r * (M / RL)) * CW + c] = v[q * RL + r];
-    __syncthreads();
-    if (bc_iv(bc)) {
-#pragma unroll
-      for (int i = 0; i < E; ++i) {
-        const int k = b + i * TPL;
-        const cplx<T> cc = cmul(xtw[M + k], buf[k * CW + c]);
-        Y(2 * k, cc.x);
-        Y(N - 1 - 2 * k, -cc.y);
+        for (int j = 0; j < E / 2; ++j) {
+          const cplx<T> Zk = v[so(j)], up = v[so(E - 1 - j)];
+          cplx<T> Zmk = {__shfl_xor_sync(0xffffffffu, up.x, 16), __shfl_xor_sync(0xffffffffu, up.y, 16)};
+          if (wi == 0) Zmk = hb ? up : (j == 0 ? Zk : v[so((E - j) % E)]);
+          pair_out(b + 32 * j, Zk, Zmk, false);
+        }
+        if (b == 0) pair_out(M / 2, v[so(E / 2)], v[so(E / 2)], true);
       }
     } else {
-      constexpr int NP = (M / 2) / TPL + 1;
+      // through the buffer
+      __syncthreads();
 #pragma unroll
-      for (int i = 0; i < NP; ++i) {
-        const int k = b + i * TPL;
-        if (k > M / 2) break;
-        const cplx<T> Zk = buf[k * CW + c], Zmk = buf[(k == 0 ? 0 : M - k) * CW + c];
-        cplx<T> Vk, Vmk;
-        if (i == NP - 1) {  // k = M/2 is its own partner
-          Vk = Vmk = cscale(conj_(Zk), (T)2 * h);
-        } else {
-          const cplx<T> Ek = cadd(Zk, conj_(Zmk));
-          const cplx<T> Ok = mul_mi(csub(Zk, conj_(Zmk)));
-          const cplx<T> B = cmul(ptw[k], Ok);
-          Vk = split_add(Ek, B, h);
-          Vmk = conj_(split_sub(Ek, B, h));
+      for (int q = 0; q < E / RL; ++q)
+#pragma unroll
+        for (int r = 0; r < RL; ++r) buf[(b + q * TPL + r * (M / RL)) * CW + c] = v[q * RL + r];
+      __syncthreads();
+      if (bc_iv(bc)) {
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+          const int k = b + i * TPL;
+          const cplx<T> cc = cmul(xtw[M + k], buf[k * CW + c]);
+          Y(2 * k, cc.x);
+          Y(N - 1 - 2 * k, -cc.y);
         }
-        if (bc == BC_P) {
-          if (k == 0) {
-            Y(0, Vk.x);
-            Y(N - 1, Vmk.x);
-          } else {
-            Y(2 * k - 1, Vk.x);
-            Y(2 * k, -Vk.y);
-            if (2 * k != M) {
-              Y(2 * (M - k) - 1, Vmk.x);
-              Y(2 * (M - k), -Vmk.y);
-            }
-          }
-        } else {
-          const bool rev = (bc == BC_DD);
-          auto OUTQ = [&](int q, T val) { Y(rev ? (N - 1 - q) : q, val); };
-          if (k == 0) {
-            OUTQ(0, Vk.x);
-            OUTQ(M, (T)0.70710678118654752440 * Vmk.x);
-          } else {
-            const cplx<T> c1 = cmul(xtw[k], Vk);
-            OUTQ(k, c1.x);
-            OUTQ(N - k, -c1.y);
-            if (2 * k != M) {
-              const cplx<T> c2 = cmul(xtw[M - k], Vmk);
-              OUTQ(M - k, c2.x);
-              OUTQ(M + k, -c2.y);
-            }
-          }
+      } else {
+        constexpr int NP = (M / 2) / TPL + 1;
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+          const int k = b + i * TPL;
+          if (k > M / 2) break;
+          const cplx<T> Zk = buf[k * CW + c], Zmk = buf[(k == 0 ? 0 : M - k) * CW + c];
+          pair_out(k, Zk, Zmk, i == NP - 1);
         }
       }
     }
   } else {
-    // ---- backward pre-processing from the rows into the buffer ----
+    // ---- backward pre-processing from the rows into the first stage's operands ----
     if (bc_iv(bc)) {
 #pragma unroll
       for (int i = 0; i < E; ++i) {
         const int k = b + i * TPL;
-        buf[k * CW + c] = cmul(cplx<T>{X(2 * k), X(N - 1 - 2 * k)}, xtw[k]);
+        const cplx<T> z = cmul(cplx<T>{X(2 * k), X(N - 1 - 2 * k)}, xtw[k]);
+        if constexpr (PAIR) v[i] = z;
+        else buf[k * CW + c] = z;
       }
     } else {
       // all row loads of the pairs first (they are independent), then the arithmetic
@@ -807,14 +845,35 @@ __device__ __forceinline__ void col_tile(const FastArgs<T>& a, const cplx<T>* st
         cplx<T> wn = ptw[k];
         wn.y = -wn.y;
         const cplx<T> Ok = cmul(csub(Vk, conj_(Vm)), wn);
-        buf[k * CW + c] = split_add(Ek, mul_i(Ok), h);
-        if (k != 0) buf[(M - k) * CW + c] = split_add(conj_(Ek), mul_i(conj_(Ok)), h);
+        const cplx<T> zk = split_add(Ek, mul_i(Ok), h), zm = split_add(conj_(Ek), mul_i(conj_(Ok)), h);
+        if constexpr (PAIR) {
+          v[i] = zk;
+          v[E - 1 - i] = zm;  // the partner's slot, exchanged below
+        } else {
+          buf[k * CW + c] = zk;
+          if (k != 0) buf[(M - k) * CW + c] = zm;
+        }
       }
-      if (b == 0) buf[(M / 2) * CW + c] = cscale(conj_(V(M / 2, xs[0], xs[1])), (T)2 * h);
-    }
-    __syncthreads();
+      const cplx<T> zh = cscale(conj_(V(M / 2, xs[0], xs[1])), (T)2 * h);  // (b = 0)
+      if constexpr (PAIR) {
+        if (wi != 0) {
 #pragma unroll
-    for (int r = 0; r < E; ++r) v[r] = buf[(b + r * TPL) * CW + c];
+          for (int i = E / 2; i < E; ++i)
+            v[i] = {__shfl_xor_sync(0xffffffffu, v[i].x, 16), __shfl_xor_sync(0xffffffffu, v[i].y, 16)};
+        } else if (hb == 0) {  // own slots: M − k of slot i is slot E − i
+#pragma unroll
+          for (int i = E - 1; i > E / 2; --i) v[i] = v[i - 1];
+          v[E / 2] = zh;
+        }
+      } else if (b == 0) {
+        buf[(M / 2) * CW + c] = zh;
+      }
+    }
+    if constexpr (!PAIR) {
+      __syncthreads();
+#pragma unroll
+      for (int r = 0; r < E; ++r) v[r] = buf[(b + r * TPL) * CW + c];
+    }
     if (bc_iv(bc)) fft_col<T, M, CW, false, 0, 1>(v, buf, stw, b, c);
     else fft_col<T, M, CW, true, 0, 1>(v, buf, stw, b, c);
     // ---- backward post-processing straight from the last stage to the rows ----
