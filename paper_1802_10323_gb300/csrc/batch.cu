@@ -581,7 +581,9 @@ ps_status build_tables(ps_batch* b) {
   if (!b->d_grids || !b->d_tasks || !b->d_stype || !b->d_sit)
     return bfail(b, PS_CUDA_ERROR, "copy of batch tables failed");
   if (b->smem > 200 * 1024) return bfail(b, PS_UNSUPPORTED_SIZE, "batch grids too large for one CTA's tiles");
-  e = cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem);
+  // (the limit is the kernel's, not the batch's: the same value for all, so that no batch lowers
+  // it under another one's launch)
+  e = cudaFuncSetAttribute(batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   if (e != cudaSuccess) return bfail(b, PS_CUDA_ERROR, "cudaFuncSetAttribute (batch kernel)");
   int bps = 0, dev_id = 0, sms = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, batch_kernel, 256, b->smem);

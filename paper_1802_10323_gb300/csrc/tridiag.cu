@@ -338,7 +338,8 @@ cudaError_t launch_zsolve64(ZArgs<double> a, cudaStream_t st) {
 cudaError_t launch_zsingular(ZArgs<float> a, cudaStream_t st) {
   const size_t smem = 2 * (size_t)a.nz * sizeof(float2);
   auto k = zsingular_kernel;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // (for n_z = 8192, whatever this plan takes: another thread may set it before this launch)
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * 8192 * (int)sizeof(float2));
   if (e != cudaSuccess) return e;
   return launch_k(k, 1, 32, smem, st, a);
 }

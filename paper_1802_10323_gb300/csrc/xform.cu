@@ -83,7 +83,8 @@ cudaError_t launch_xform(XformArgs<T> a, cudaStream_t st) {
   int threads = (((a.m << lg) / 8 + 31) / 32) * 32;
   threads = threads < 64 ? 64 : (threads > 256 ? 256 : threads);
   auto k = xform_kernel<T, TI, TO, FWD>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the most a block may have, whatever this tile takes: another thread may set it before this launch
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
   if (e != cudaSuccess) return e;
   return launch_k(k, (unsigned)tiles(lg), threads, smem, st, a);
 }
