@@ -82,15 +82,19 @@ typedef enum {
  *   PS_FP32_REFINE  FP64 fields; FP32 bulk transforms and tridiagonal solves,
  *                   iterative refinement whose residual r = f − A·Φ is formed
  *                   in double-float (pairs of FP32) from the FP64 fields, until
- *                   ‖r‖∞ ≤ rtol·‖f_c‖∞ or max_iter corrections (the first correction
- *                   ends it at half of rtol while another is allowed). */
+ *                   ‖r‖∞ ≤ rtol·‖f_c‖∞ or max_iter corrections. A plan's solve whose
+ *                   first correction ends in (rtol/2, rtol] makes one more where
+ *                   max_iter allows it and rtol is well above the rounding of p,
+ *                   and takes it back if it missed rtol; the batched solve ends
+ *                   each grid at rtol. */
 typedef enum { PS_FP64 = 0, PS_FP32 = 1, PS_FP32_REFINE = 2 } ps_precision;
 
 /* Device-side record written by every solve (caller allocates it in device
  * memory; read it after synchronising the stream). */
 typedef struct {
   int status;             /* ps_status of the device work (OK, NOT_CONVERGED, TIMEOUT) */
-  int iterations;         /* refinement corrections applied (0 for FP64 / FP32)        */
+  int iterations;         /* refinement corrections made (0 for FP64 / FP32), a       */
+                          /* second one that was taken back included                  */
   double rel_residual;    /* ‖f_c − A·Φ‖∞ / ‖f_c‖∞ measured on the device (refine);   */
                           /* −1 when not measured (FP64 / FP32 modes)                  */
   double r_norm;          /* ‖f_c − A·Φ‖∞ (refine), else −1                            */

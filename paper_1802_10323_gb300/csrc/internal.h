@@ -176,15 +176,18 @@ struct Ctrl {
   int skip_redo;            // 0: pass 0 is repeated with the three-level split
   int nomat0;               // 0: the loop ended at pass 0, p is written from Φ_0
   int skip_out;             // 0: a pass m ≥ 1 found no convergence; it is repeated with its output
-  int pad2;
+  int met;                  // 1: the first correction reached rtol and another one was asked for
   unsigned long long dmax_prev;  // max|e| of the correction the current pass used
+  double rel1, rnorm1;      // the first correction's residual when met is set
+  int undo;                 // 1: the second correction missed rtol after met; it is taken back from p
 };
 
 cudaError_t launch_finalize(Ctrl* ctrl, const float* partial, int nblocks, double wsum_total,
                             int singular, double rtol, int iteration, int attempt, int last,
                             double anorm, const int* skip, ps_info* info, cudaStream_t st);
-// p = Φ_0 (widened exactly) unless *skip.
-cudaError_t launch_widen(const float* u, double* p, size_t n, const int* skip, cudaStream_t st);
+// After the loop: p = Φ_0 (widened exactly) if it ended at pass 0; p −= e if the second
+// correction is taken back (Ctrl::undo); else nothing.
+cudaError_t launch_settle(const float* u0, const float* e, double* p, size_t n, const Ctrl* ctrl, cudaStream_t st);
 cudaError_t launch_finalize_exact(Ctrl* ctrl, const float* partial, int nblocks, double wsum_total,
                                   int singular, double rtol, ps_info* info, cudaStream_t st);
 cudaError_t launch_info_plain(ps_info* info, cudaStream_t st);

@@ -788,9 +788,6 @@ ps_status solve_refine(ps_plan* pl, const double* f, double* p, void* ws, cudaSt
                                     pl->rtol, 0, 1, last ? 1 : 0, pl->anorm, &ctrl->skip_redo, info, st);
            })) != cudaSuccess)
         return cuda_fail(pl, e, "finalize");
-      // the loop ended at pass 0 (converged or max_iter = 0): p = Φ_0
-      if ((e = run(pl, K_MAT, st, [&] { return launch_widen(u0, p, pl->N, &ctrl->nomat0, st); })) != cudaSuccess)
-        return cuda_fail(pl, e, "store");
     }
     if (it > 0 && !last) {  // the output repeat of pass it, only if it did not converge
       ResidArgs ro = ra;
@@ -803,6 +800,10 @@ ps_status solve_refine(ps_plan* pl, const double* f, double* p, void* ws, cudaSt
     }
     if (!last && (e = correction(it + 1)) != cudaSuccess) return cuda_fail(pl, e, "correction");
   }
+  // the loop ended at pass 0 (converged or max_iter = 0): p = Φ_0; or its second correction
+  // is taken back: p −= e (in w since pass 2, nothing having run after it)
+  if ((e = run(pl, K_MAT, st, [&] { return launch_settle(u0, w, p, pl->N, ctrl, st); })) != cudaSuccess)
+    return cuda_fail(pl, e, "store");
   // Exact confirmation from the stored p, only when the drift bound of the
   // incremental passes was not small (both kernels return at once otherwise).
   ResidArgs rx = ra;
