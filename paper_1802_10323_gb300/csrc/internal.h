@@ -38,6 +38,7 @@ __host__ __device__ inline bool bc_iv(int bc) { return bc == BC_ND || bc == BC_D
 // kernels; longer ones in the shared-memory kernel, one line per CTA (two buffers
 // of n/2 + 1 complex values: 131 KB for an FP64 line of 8192)
 constexpr int kMaxN = 8192;
+constexpr int kSMs = 152;  // of the part this is written for (rules on how far work is split)
 constexpr int kMaxStages = 6;   // of a generic line FFT (radices up to 9: m ≤ 4096 needs 4)
 extern thread_local char g_launch_diag[256];  // configuration of the last failed launch
 // Test hook (ps_inject_alloc_failures): true while injected device-allocation failures

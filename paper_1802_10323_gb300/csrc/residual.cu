@@ -850,7 +850,7 @@ ResidShape resid_shape(int nx, int ny, int nz, int which) {
         : (which == RS_ACC && ny >= 8 * RWARPS) ? 8 : (ny >= 4 * RWARPS ? 4 : 2);
   const int tiles = ((nx + RTX - 1) / RTX) * ((ny + RWARPS * s.rpt - 1) / (RWARPS * s.rpt));
   // about four waves of three CTAs per SM, 8 … 64 planes per CTA
-  const long long want = 152LL * (s.rpt >= 8 ? 2 : 3) * 4;
+  const long long want = (long long)kSMs * (s.rpt >= 8 ? 2 : 3) * 4;
   long long zc = ((long long)nz * tiles) / want;
   zc = zc < 8 ? 8 : (zc > 64 ? 64 : zc);
   s.zchunk = (int)(zc < nz ? zc : nz);
@@ -1181,7 +1181,7 @@ __global__ void settle_kernel(const float* __restrict__ u0, const float* __restr
 }
 
 cudaError_t launch_settle(const float* u0, const float* e, double* p, size_t n, const Ctrl* ctrl, cudaStream_t st) {
-  return launch_k(settle_kernel, 152 * 8, 256, 0, st, u0, e, p, n, ctrl);
+  return launch_k(settle_kernel, kSMs * 8, 256, 0, st, u0, e, p, n, ctrl);
 }
 
 __global__ void info_plain_kernel(ps_info* info) {

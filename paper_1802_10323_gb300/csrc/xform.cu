@@ -26,7 +26,7 @@ template <class TI, class TO, int AXIS, bool FWD, int M>
 cudaError_t mid_case(const XformArgs<float>& a, cudaStream_t st, bool* done) {
   const int L = mid::DimCt<M>::L;
   const long long tiles = AXIS == 0 ? (a.nlines + L - 1) / L : (long long)a.nz * ((a.nx + L - 1) / L);
-  if (tiles < 152) return cudaSuccess;
+  if (tiles < kSMs) return cudaSuccess;
   *done = true;
   return launch_xform_mid<TI, TO, M, AXIS, FWD>(a, (int)tiles, st);
 }
@@ -53,8 +53,13 @@ cudaError_t launch_mid_if(const XformArgs<float>& a, cudaStream_t st, bool* done
 
 // Lines per tile: 16 (a 64-byte row segment of FP32 y lines, full half-warps) while four
 // CTAs fit an SM (56 KB each); fewer on long lines, down to four (FP32: one 16-byte part of
-// a sector) as long as a CTA's shared memory holds them; and fewer, down to four, while the
-// tiles would leave SMs without work: on a 32^3 grid 16 lines make 64 tiles, four make 256.
+// a sector), and below that where only one such CTA would fit an SM (its 256 threads then
+// wait out every load and FP64 chain alone: 4000 FP32 x lines of 4608, forward and backward,
+// µs, with 4, 2 and 1 lines: 463, 329 and 254, of 7776 with 2 and 1: 946 and 454; 1400 FP64
+// lines of 2592 with 4, 2 and 1: 541, 517 and 440); and fewer, down to four, while the tiles
+// would leave SMs without work: on a 32^3 grid 16 lines make 64 tiles, four make 256. A tile
+// of long lines (486 points or more) may go on to one line (24 FP64 x lines of 2592 with 4, 2
+// and 1 lines: 185, 114 and 69 µs).
 template <class T, class TI, class TO, bool FWD>
 cudaError_t launch_xform(XformArgs<T> a, cudaStream_t st) {
   if constexpr (sizeof(T) == 4) {
@@ -68,15 +73,15 @@ cudaError_t launch_xform(XformArgs<T> a, cudaStream_t st) {
     if (e != cudaSuccess || done) return e;
   }
   constexpr size_t C = sizeof(cplx<T>);
-  constexpr size_t kBest = 56 * 1024, kMost = 220 * 1024;
+  constexpr size_t kBest = 56 * 1024, kTwo = 110 * 1024;  // four and two CTAs an SM
   auto tiles = [&](int lg) -> long long {
     const int L = 1 << lg;
     return a.axis == 0 ? (a.nlines + L - 1) / L : (long long)a.nz * ((a.nx + L - 1) / L);
   };
   int lg = 4;
   while (lg > 2 && tile_smem(a.m, lg, C) > kBest) --lg;
-  while (lg > 0 && tile_smem(a.m, lg, C) > kMost) --lg;
-  while (lg > 2 && tiles(lg) < 2 * 152) --lg;
+  while (lg > 0 && tile_smem(a.m, lg, C) > kTwo) --lg;
+  while (lg > 0 && tiles(lg) < 2 * kSMs && (lg > 2 || (a.m << lg) >= 486)) --lg;
   a.lgL = lg;
   const size_t smem = tile_smem(a.m, lg, C);
   // a thread per eight points of the tile, in whole warps
