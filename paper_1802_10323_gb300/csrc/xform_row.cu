@@ -23,10 +23,10 @@
 namespace ps {
 namespace row {
 
-template <class T, class TI, class TO, int M, bool FWD, int OM>
+template <class T, class TI, class TO, int M, bool FWD, int OM, bool W>
 __global__ void __launch_bounds__(32 * kWarps<T>, sizeof(T) == 4 ? (M >= 512 ? 3 : 4) : 3)
     xform_row_kernel(FastArgs<T> a) {
-  constexpr int LPW = 32 / Shape<M, kWide<T>>::TPL;
+  constexpr int LPW = 32 / Shape<M, W>::TPL;
   constexpr int LB = M + M / 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cplx<T>* stw = reinterpret_cast<cplx<T>*>(smem_raw);
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(32 * kWarps<T>, sizeof(T) == 4 ? (M >= 512 ? 3
   T tmax = (T)0;
   const int wstride = gridDim.x * kWarps<T> * LPW;
   for (int l0 = (blockIdx.x * kWarps<T> + warp) * LPW; l0 < a.nlines; l0 += wstride)
-    row_line<T, TI, TO, M, FWD, OM>(a, stw, ptw, xtw, bufs + warp * LPW * LB, l0, tmax);
+    row_line<T, TI, TO, M, FWD, OM, W>(a, stw, ptw, xtw, bufs + warp * LPW * LB, l0, tmax);
   if constexpr (sizeof(TO) == 8) {
     if (a.amax) {
       for (int o = 16; o > 0; o >>= 1) tmax = fmax(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
@@ -57,12 +57,12 @@ __global__ void __launch_bounds__(32 * kWarps<T>, sizeof(T) == 4 ? (M >= 512 ? 3
 }  // namespace row
 
 namespace {
-template <class T, class TI, class TO, int M, bool FWD, int OM>
-cudaError_t launch_row_mode(FastArgs<T> a, cudaStream_t st) {
-  using S = fast::Shape<M, row::kWide<T>>;
+template <class T, class TI, class TO, int M, bool FWD, int OM, bool W>
+cudaError_t launch_row_shape(FastArgs<T> a, cudaStream_t st) {
+  using S = fast::Shape<M, W>;
   constexpr int LPW = 32 / S::TPL;
   constexpr size_t LB = M + M / 8;
-  auto k = row::xform_row_kernel<T, TI, TO, M, FWD, OM>;
+  auto k = row::xform_row_kernel<T, TI, TO, M, FWD, OM, W>;
   const size_t smem = fast_table_bytes<T, M>(a.bc) + (size_t)row::kWarps<T> * LPW * LB * sizeof(cplx<T>);
   static int smem_set = 0;
   static int blocks_per_sm[2] = {};
@@ -86,6 +86,13 @@ cudaError_t launch_row_mode(FastArgs<T> a, cudaStream_t st) {
   const int grid = ctas < sms * bps ? ctas : sms * bps;
   (void)cudaGetLastError();  // a stale error from elsewhere must not be blamed here
   return launch_k(k, grid, 32 * row::kWarps<T>, smem, st, a);
+}
+template <class T, class TI, class TO, int M, bool FWD, int OM>
+cudaError_t launch_row_mode(const FastArgs<T>& a, cudaStream_t st) {
+  if constexpr (sizeof(T) == 8 && M < 512) {
+    if (a.nlines <= row::kFewLines) return launch_row_shape<T, TI, TO, M, FWD, OM, false>(a, st);
+  }
+  return launch_row_shape<T, TI, TO, M, FWD, OM, row::kWide<T>>(a, st);
 }
 }  // namespace
 

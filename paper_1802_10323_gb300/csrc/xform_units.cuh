@@ -73,6 +73,12 @@ template <class T>
 constexpr int kWarps = sizeof(T) == 8 ? 4 : 8;
 template <class T>
 constexpr bool kWide = sizeof(T) == 8;
+// FP64 passes of at most this many lines (two per SM sub-partition) take the narrow stages:
+// there a pass is one warp's chain of FP64 instructions, which a wide warp's four lines
+// (M = 128) make four times longer. Forward passes, periodic, µs, wide and narrow: n = 256,
+// 512 lines 25.5 and 14.6, 1024 lines 26.1 and 17.7, 2048 lines 26.2 and 27.0; n = 512,
+// 512 lines 27.4 and 18.8, 1024 lines 28.5 and 27.3, 2048 lines 44.5 and 45.6.
+constexpr int kFewLines = 1216;
 
 template <class TC, class TI>
 __device__ __forceinline__ TC in_cvt(TI x) { return ld_cvt<TC, TI>::f(x); }
@@ -109,10 +115,9 @@ struct LaneSlots {
 // exchange buffers at bufs, tables in shared memory, the first line index l0.
 // tmax accumulates max |FP64 output| for the caller's reduction (before widening; FP64
 // transforms only when asked: the comparison costs their pipe).
-template <class T, class TI, class TO, int M, bool FWD, int OM>
+template <class T, class TI, class TO, int M, bool FWD, int OM, bool W>
 __device__ __forceinline__ void row_line(const FastArgs<T>& a, const cplx<T>* stw, const cplx<T>* ptw,
                                          const cplx<T>* xtw, cplx<T>* bufs, int l0, T& tmax) {
-  constexpr bool W = kWide<T>;
   using S = Shape<M, W>;
   constexpr int N = 2 * M, E = S::E, TPL = S::TPL;
   constexpr int R0 = S::radix(0), RL = S::radix(S::NST - 1);

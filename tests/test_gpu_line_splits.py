@@ -1,7 +1,8 @@
 """The line transforms on both sides of the rules that split a pass over the chip.
 
-Lines whose length is no power of two run in tiles of four, two or one, by their length and
-number. Against the oracle, with the tolerances of the solver's other
+FP64 x passes of power-of-two lines change their stages at 1216 lines (the passes beyond leave
+the last warp with two of its four lines); lines of other lengths run in tiles of four, two or
+one, by their length and number. Against the oracle, with the tolerances of the solver's other
 parity tests: FP64 1e-12, the refined solve 1e-9 (rtol 1e-10) and FP32 5e-5 of ‖p‖∞.
 """
 
@@ -14,7 +15,9 @@ from paper_1802_10323_gb300 import synth
 pytestmark = pytest.mark.gpu
 
 ALL = ("fp64", "fp32", "fp32_refine")
-CASES = [(1296, 54, 7, "NN", "DD", ALL),    # 378 rows of 648 points
+CASES = [(n, 64, 19, b, "P", ("fp64",)) for n, b in ((128, "DD"), (256, "P"), (512, "ND"))] + \
+        [(n, 6, 203, b, "P", ("fp64",)) for n, b in ((128, "DN"), (256, "NN"), (256, "DD"), (512, "P"))] + \
+        [(1296, 54, 7, "NN", "DD", ALL),    # 378 rows of 648 points
          (1296, 54, 23, "DN", "P", ALL),    # 1242
          (12, 1944, 3, "P", "ND", ALL),     # columns of 972 points, one each
          (108, 2592, 6, "NN", "DD", ALL),   # 648 columns of 1296
