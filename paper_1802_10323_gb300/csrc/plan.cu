@@ -17,6 +17,7 @@
 #include <type_traits>
 
 #include "internal.h"
+#include "low_rect.h"
 #include "xform_fast.cuh"
 
 using namespace ps;
@@ -1050,34 +1051,15 @@ ps_status ps_plan_create_helmholtz(ps_plan** out, int nx, int ny, int nz, double
   p->dev = dev;
   size_t off = 0;
   {
-    // FP32 paths: columns whose z system has κ ≈ ‖T_z‖/|λ| above a limit are solved in
-    // double-float (tridiag.cu; a periodic z needs 32 planes for that). λ grows with q along
-    // each axis, so they lie in the rectangle q_x < lowx, q_y < lowy; at most 1/8 of the
-    // columns. A Helmholtz shift adds α to every |λ| (all terms of the diagonal shift have one
-    // sign). The limit is 10^5, or 10^3 where that makes at most two columns an SM, which run
-    // beside the FP32 columns: on thin or coarse grids the lowest modes carry the solution,
-    // and a column's FP32 error is about ε·κ (4096×4096×16
-    // after one correction: 1.2e-9 with 10^5 alone, 5–6e-10; the z pass keeps its 387 µs).
+    // FP32 paths: columns whose z system has the largest κ ≈ ‖T_z‖/|λ| are solved in
+    // double-float (tridiag.cu; a periodic z needs 32 planes for that). A Helmholtz shift adds
+    // α to every |λ| (all terms of the diagonal shift have one sign).
     p->lowx = p->lowy = 0;
     if (prec != PS_FP64 && (bcz != PS_BC_PERIODIC || nz >= 32)) {
       double zmax = 0.0;
       for (int k = 0; k < nz; ++k)
         zmax = std::max(zmax, std::fabs(za[k]) + std::fabs(zb[k]) + std::fabs(zc[k]));
-      const std::vector<double> lx = eig_scaled(bcx, nx, dx), ly = eig_scaled(bcy, ny, dy);
-      for (const double limit : {1e3, 1e5}) {
-        p->lowx = p->lowy = 0;
-        const double thr = zmax / limit;
-        int qx = 0, qy = 0;
-        while (qx < nx && std::fabs(lx[qx]) + alpha < thr) ++qx;
-        while (qy < ny && std::fabs(ly[qy]) + alpha < thr) ++qy;
-        while ((size_t)qx * qy * 8 > (size_t)nx * ny && qy > 1) --qy;
-        while ((size_t)qx * qy * 8 > (size_t)nx * ny && qx > 1) --qx;
-        if ((size_t)qx * qy * 8 <= (size_t)nx * ny && qx > 0 && qy > 0) {
-          p->lowx = qx;
-          p->lowy = qy;
-        }
-        if (p->lowx * p->lowy <= 304) break;
-      }
+      low_rectangle(eig_scaled(bcx, nx, dx), eig_scaled(bcy, ny, dy), alpha, zmax, 2 * kSMs, &p->lowx, &p->lowy);
     }
   }
   auto take = [&](size_t nbytes) { char* q = dev + off; off += align256(nbytes); return q; };

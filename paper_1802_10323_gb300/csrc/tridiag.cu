@@ -40,8 +40,8 @@ constexpr int ZTAB_MAX = 4096;     // planes whose coefficient table sits in sha
 // stretched channel grid. The elimination in excess form keeps λ's digits, but the FP32
 // sums over the right-hand side still err by up to ~√n_z·ε_32 of Σ|f̂|/|λ|, smooth in z
 // with a large amplitude: what an FP32 correction solve removes worst. The columns with
-// κ > 10^5 (10^3 where that makes at most two columns an SM; plan.cu) — a rectangle
-// q_x < lowx, q_y < lowy fixed at plan creation — are solved here
+// the largest κ — a rectangle q_x < lowx, q_y < lowy fixed at plan creation (low_rect.h:
+// κ > 10^5 in any case, down to 10^3 while two columns an SM are enough) — are solved here
 // in double-float arithmetic, ~2^−46 relative per operation against ε_32 = 2^−24 (the
 // singular column (0,0) with its weighted-mean pinning among them), by CTAs of the same
 // launch as the FP32 columns, so they overlap them. Output rounded to FP32. (The line:
