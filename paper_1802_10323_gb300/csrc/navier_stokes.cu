@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(PTX * PTY, PMINB) ns_predict_kernel(NsArgs<T> 
 }
 
 // p += Φ'/(γΔt), and Φ' → Φ in place (2d), in 16-byte pieces (the substep's arrays are
-// 16-byte aligned; n_x is even, and the FP32 tail of N mod 4 = 2 values is taken singly)
+// 16-byte aligned; n_x and n_y are even, so that N is a multiple of four)
 template <class T>
 __global__ void __launch_bounds__(256) ns_pressure_kernel(size_t N, T scale, T* __restrict__ p,
                                                           T* __restrict__ phi) {
@@ -287,11 +287,6 @@ __global__ void __launch_bounds__(256) ns_pressure_kernel(size_t N, T scale, T* 
     }
     reinterpret_cast<Vec*>(phi)[g] = f;
     reinterpret_cast<Vec*>(p)[g] = q;
-  }
-  for (size_t g = NV * V + t; g < N; g += stride) {
-    const T f = phi[g] * scale;
-    phi[g] = f;
-    p[g] += f;
   }
 }
 
