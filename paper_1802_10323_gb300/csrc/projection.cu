@@ -23,8 +23,8 @@ namespace ps {
 // ProjArgs (internal.h): per[] = axis periodic; idx, idy = 1/Δx, 1/Δy; idzf[k] = 1/Δz^f_k;
 // idzc[k] = 1/(centre distance between cells k−1 and k), idzc[0] = the periodic wrap.
 
-// A row (j, k) per group of threadIdx.x, V consecutive cells a thread (16-byte accesses when
-// n_x and the pointers allow, else V = 1): the ends of y and z are decided once per row, those
+// A row (j, k), or on few rows a part of one, per group of threadIdx.x, V consecutive cells a
+// thread (16-byte accesses when n_x and the pointers allow, else V = 1): the ends of y and z are decided once per row, those
 // of x for one cell of it, and no cell pays a division. The fused multiply-adds are written out:
 // both widths then give the same bits. Bound by HBM in FP32 and by the FP64
 // pipe in FP64 (6 instructions a cell and kernel, 627 G/s on this part). Measured on
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(256) div_kernel(ProjArgs<T> a, const T* __rest
   const T* __restrict__ uy = u + N + r.base;
   const T* __restrict__ uz = u + 2 * N + r.base;
   const T idz = a.idzf[r.k];
-  for (int i = threadIdx.x * V; i < a.nx; i += blockDim.x * V) {
+  for (int i = (blockIdx.y * blockDim.x + threadIdx.x) * V; i < a.nx; i += gridDim.y * blockDim.x * V) {
     const auto x = ld_cells<T, V>(ux + i), yl = ld_cells<T, V>(uy + i), zl = ld_cells<T, V>(uz + i);
     const auto yh = ld_cells<T, V>(uy + r.yp + i), zh = ld_cells<T, V>(uz + r.zp + i);
     const T xn = (i + V < a.nx) ? ux[i + V] : (a.per[0] ? ux[0] : (T)0);
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(256) grad_correct_kernel(ProjArgs<T> a, const 
   const size_t N = (size_t)a.nx * a.ny * a.nz;
   const T* __restrict__ p = phi + r.base;
   const T idz = a.idzc[r.k];
-  for (int i = threadIdx.x * V; i < a.nx; i += blockDim.x * V) {
+  for (int i = (blockIdx.y * blockDim.x + threadIdx.x) * V; i < a.nx; i += gridDim.y * blockDim.x * V) {
     const auto pc = ld_cells<T, V>(p + i), py = ld_cells<T, V>(p + r.ym + i), pz = ld_cells<T, V>(p + r.zm + i);
     const bool hxm = i > 0 || a.per[0];
     const T px = i > 0 ? p[i - 1] : (a.per[0] ? p[a.nx - 1] : (T)0);
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(256) grad_adjoint_kernel(ProjArgs<T> a, const 
   const T* __restrict__ gy = gu + N + r.base;
   const T* __restrict__ gz = gu + 2 * N + r.base;
   const T dl = a.idzc[r.k], dh = a.idzc[r.k + 1 < a.nz ? r.k + 1 : 0];
-  for (int i = threadIdx.x * V; i < a.nx; i += blockDim.x * V) {
+  for (int i = (blockIdx.y * blockDim.x + threadIdx.x) * V; i < a.nx; i += gridDim.y * blockDim.x * V) {
     const auto x = ld_cells<T, V>(gx + i), yl = ld_cells<T, V>(gy + i), zl = ld_cells<T, V>(gz + i);
     const auto yh = ld_cells<T, V>(gy + r.yp + i), zh = ld_cells<T, V>(gz + r.zp + i);
     const bool hxp = i + V < a.nx || a.per[0];
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(256) div_adjoint_correct_kernel(ProjArgs<T> a,
   const size_t N = (size_t)a.nx * a.ny * a.nz;
   const T* __restrict__ s = s_ + r.base;
   const T wm = a.idzf[r.k > 0 ? r.k - 1 : a.nz - 1], wc = a.idzf[r.k];
-  for (int i = threadIdx.x * V; i < a.nx; i += blockDim.x * V) {
+  for (int i = (blockIdx.y * blockDim.x + threadIdx.x) * V; i < a.nx; i += gridDim.y * blockDim.x * V) {
     // face i lies between cell i−1 (contributes s/Δ) and cell i (−s/Δ)
     const auto sc = ld_cells<T, V>(s + i), sy = ld_cells<T, V>(s + r.ym + i), sz = ld_cells<T, V>(s + r.zm + i);
     const bool hxm = i > 0 || a.per[0];
@@ -189,7 +189,12 @@ cudaError_t launch_op(int op, const ProjArgs<T>& a, const T* a0, const T* a1, T*
   int tx = 1;  // threads of a row: a power of two, a warp at most
   while (tx < 32 && tx * V < a.nx) tx *= 2;
   const dim3 block(tx, 256 / tx);
-  const unsigned grid = (unsigned)(((long long)a.ny * a.nz + block.y - 1) / block.y);
+  const unsigned rows = (unsigned)(((long long)a.ny * a.nz + block.y - 1) / block.y);
+  // rows too few for eight CTAs an SM are cut along x, down to one vector a thread: a thread's
+  // vectors are a chain of load latencies (FP64 divergence and gradient of 3072×4×2, µs: 98 in one
+  // part, 13 in parts)
+  const unsigned parts = (unsigned)((a.nx + tx * V - 1) / (tx * V)), want = 8 * kSMs / rows;
+  const dim3 grid(rows, want < 1 ? 1 : (want < parts ? want : parts));
   switch (op) {
     case 0: return launch_k(div_kernel<T, V>, grid, block, 0, st, a, a0, o);
     case 1: return launch_k(grad_correct_kernel<T, V>, grid, block, 0, st, a, a0, a1, o);
