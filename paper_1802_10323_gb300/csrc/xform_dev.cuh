@@ -281,7 +281,7 @@ template <class D, class T, class TI, bool FWD, class Scale>
 __device__ __forceinline__ void x_load(const D& d, int bc, const TI* in, int live, T* rA, bool scaled, Scale&& scale_of) {
   const int m = d.m(), ls = d.ls();
   const bool al = !((uintptr_t)in & (2 * sizeof(TI) - 1));
-  const T sg = (FWD && bc == BC_DD) ? (T)-1 : (T)1;  // DST ordering: the odd elements change sign
+  const bool neg = FWD && bc == BC_DD;  // DST ordering: the odd elements change sign
   by_kind(bc, [&](auto kind) {
     constexpr int KIND = decltype(kind)::value;
     const SlotMap<D, KIND> map{d, bc};
@@ -303,7 +303,7 @@ __device__ __forceinline__ void x_load(const D& d, int bc, const TI* in, int liv
         if (FWD) map.phys_of(e, s0, c0, s1, c1);
         else map.spec_of(e, s0, c0, s1, c1);
         rA[2 * (s0 * ls + l) + c0] = v0;
-        rA[2 * (s1 * ls + l) + c1] = (FWD && KIND == KIND_CT) ? sg * v1 : v1;
+        rA[2 * (s1 * ls + l) + c1] = (FWD && KIND == KIND_CT && neg) ? -v1 : v1;
       }
     }
   });
@@ -373,7 +373,7 @@ template <class D, class T, class TO, bool FWD, class Args, class Scale>
 __device__ __forceinline__ void x_store(const D& d, const Args& a, TO* out, size_t base, int live, const T* rS, int sw,
                                         bool fd, bool scaled, Scale&& scale_of, T& tmax) {
   const int n = d.n(), ls = d.ls(), bc = a.bc;
-  const T sg = (!FWD && bc == BC_DD) ? (T)-1 : (T)1;
+  const bool neg = !FWD && bc == BC_DD;
   const bool al = !((((uintptr_t)out) & (2 * sizeof(TO) - 1)) | (((uintptr_t)a.out2 | (uintptr_t)a.base32) & 7));
   TO* dst = out + base;
   const float* b32 = a.base32 ? a.base32 + base : nullptr;
@@ -395,7 +395,7 @@ __device__ __forceinline__ void x_store(const D& d, const Args& a, TO* out, size
         map.phys_of(e, s0, c0, s1, c1);
       }
       T v0 = rS[2 * (s0 * ls + l) + (c0 ^ sw)], v1 = rS[2 * (s1 * ls + l) + (c1 ^ sw)];
-      if constexpr (!FWD && KIND == KIND_CT) v1 *= sg;
+      if constexpr (!FWD && KIND == KIND_CT) v1 = neg ? -v1 : v1;
       if (scaled) {
         const T sc = scale_of(l);
         v0 *= sc;
@@ -493,7 +493,8 @@ __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_
       const int j = a.axis == 0 ? idx - l * m : idx >> lgL;
       if (l >= live) continue;
       const T sc = fscale ? scale_of(l) : (T)1;
-      bufA[j * ls + l] = cplx<T>{val(l, 2 * j) * sc, val(l, 2 * j + 1) * sc};
+      const cplx<T> z = {val(l, 2 * j), val(l, 2 * j + 1)};
+      bufA[j * ls + l] = fscale ? cscale(z, sc) : z;
       if (j == 0) {
         const T w = ld_cvt<T, TI>::f(a.axis == 0 ? in[base + (size_t)l * n] : in[base + l]);
         bufA[m * ls + l] = cplx<T>{w * sc, (T)0};
@@ -518,8 +519,10 @@ __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_
           if (e0 & 1) v0 = -v0;
           if (e1 & 1) v1 = -v1;
         }
-        v0 *= sc;
-        v1 *= sc;
+        if (fscale) {
+          v0 *= sc;
+          v1 *= sc;
+        }
       }
       bufA[p * ls + l] = cplx<T>{v0, v1};
     }
@@ -590,8 +593,8 @@ __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_
       int e0, e1;
       if (FWD) map.spec(k, e0, e1);
       else map.phys(k, e0, e1);
-      emit(base + (size_t)(e0 * nx) + l, FWD ? v0 : v0 * yscale);
-      emit(base + (size_t)(e1 * nx) + l, FWD ? v1 : v1 * yscale);
+      emit(base + (size_t)(e0 * nx) + l, bscale ? v0 * yscale : v0);
+      emit(base + (size_t)(e1 * nx) + l, bscale ? v1 * yscale : v1);
     }
   };
   if (fd) {  // X_k = −Im(Y_k), k = 1 … n−1 (× 1/2n backward), into part 0 of slot k
@@ -632,7 +635,7 @@ __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_
   } else if (fd) {
     for (int idx = tid; idx < (n << lgL); idx += nt) {
       const int l = idx & lm, e = idx >> lgL;
-      if (l < live) emit(base + (size_t)(e * nx) + l, rS[2 * (e * ls + l)] * yscale);
+      if (l < live) emit(base + (size_t)(e * nx) + l, bscale ? rS[2 * (e * ls + l)] * yscale : rS[2 * (e * ls + l)]);
     }
   } else if (!FWD && !iv) {
     by_kind(bc, [&](auto kind) {
@@ -644,8 +647,8 @@ __device__ void xform_group(const XformArgs<T>& a, int grp, unsigned char* smem_
       int e0, e1;
       map.phys(p, e0, e1);
       const T v0 = (bc == BC_DD && (e0 & 1)) ? -z.y : z.y, v1 = (bc == BC_DD && (e1 & 1)) ? -z.x : z.x;
-      emit(base + (size_t)(e0 * nx) + l, v0 * yscale);
-      emit(base + (size_t)(e1 * nx) + l, v1 * yscale);
+      emit(base + (size_t)(e0 * nx) + l, bscale ? v0 * yscale : v0);
+      emit(base + (size_t)(e1 * nx) + l, bscale ? v1 * yscale : v1);
     }
     });
   }
