@@ -292,14 +292,15 @@ cudaError_t launch_zsolve_ckpt(ZArgs<float> a, cudaStream_t st) {
                     : launch_ckpt<false, false, false>(a, grid, nlowb, 0, st);
 }
 
-// FP64: a thread per column; on planes of few columns, where that leaves most of the chip
+// FP64: a thread per column, or on planes of few columns, where that leaves most of the chip
 // idle behind serial chains, a warp per column. The singular column is always a warp's
-// (block 0). A warp spends about 2.5 times the FP64 instructions a thread's column takes,
-// so the line lies where a thread per column reaches 0.4 of the SM sub-partitions (8192
-// columns = 256 of 608 warps). 32^3: 32 + 22 µs (columns, singular column) → 13 µs;
-// 256^3: 564 → 429 µs (11 FP64 instructions a row instead of 20; the FP64 pipe binds, with
-// 3.4 warps per sub-partition taking the time of four).
-constexpr int ZPART_COLS = 8192;
+// (block 0). Measured, a thread's chain takes 4 + 0.61·n_z µs, and warps 7 + N·(0.003 +
+// 0.00009·n_z) µs for N columns; a warp each where that is less: n_z ≥ 12 at 1024 columns, 22 at
+// 2048, 63 at 4096, never beyond 6700. Thread and warp, µs: 32×32×32 22 and 10, 64×64×64 43 and
+// 43, 64×64×256 154 and 117, 128×64×64 41 and 67, 64×64×8 10 and 24. 256^3: 564 → 429 µs (11
+// FP64 instructions a row instead of 20; the FP64 pipe binds, with 3.4 warps per sub-partition
+// taking the time of four).
+inline bool warp_columns(int ncol, int nz) { return (6800LL - ncol) * nz > 33LL * (1000 + ncol); }
 __global__ void __launch_bounds__(128) zsolve64_kernel(ZArgs<double> a) {
   pdl_wait();
   int b = blockIdx.x;
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(32) zsingular_kernel(ZArgs<float> a) {
 
 cudaError_t launch_zsolve64(ZArgs<double> a, cudaStream_t st) {
   const int ncol = a.nx * a.ny;
-  if (ncol <= ZPART_COLS && (!a.periodic || a.nz >= 32))
+  if (warp_columns(ncol, a.nz) && (!a.periodic || a.nz >= 32))
     return launch_k(zpart64_kernel, (ncol + 3) / 4, 128, 0, st, a);
   return launch_k(zsolve64_kernel, (ncol + 127) / 128 + (a.singular ? 1 : 0), 128, 0, st, a);
 }
