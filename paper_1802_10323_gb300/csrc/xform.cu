@@ -26,12 +26,13 @@ template <class TI, class TO, int AXIS, bool FWD, int M>
 cudaError_t mid_case(const XformArgs<float>& a, cudaStream_t st, bool* done) {
   const int L = mid::DimCt<M>::L;
   const long long tiles = AXIS == 0 ? (a.nlines + L - 1) / L : (long long)a.nz * ((a.nx + L - 1) / L);
-  if (tiles < kSMs) return cudaSuccess;
+  if (tiles < kSMs || (AXIS == 1 && tiles * L > 2LL * a.nz * a.nx)) return cudaSuccess;
   *done = true;
   return launch_xform_mid<TI, TO, M, AXIS, FWD>(a, (int)tiles, st);
 }
 // FP32 lines: the kernel with the length at compile time, where the grid gives every SM a
-// tile of it (fewer tiles: the run-time kernel, whose tiles shrink with the grid).
+// tile of it and no more than half of a plane's tiles' columns are idle (else the run-time
+// kernel, whose tiles shrink with the grid: 2 columns of 972, 4096 planes: 489 → 96 µs).
 // 384×288×201 in µs, run-time → compile-time length: x 97 → 73 forward, 99 → 75 backward (into
 // FP32 Φ_0), 160 → 136 (into p), y 113 → 54 and 105 → 56; 192×96×65 solve 45 → 32.
 template <class TI, class TO, int AXIS, bool FWD>
@@ -59,7 +60,12 @@ cudaError_t launch_mid_if(const XformArgs<float>& a, cudaStream_t st, bool* done
 // lines of 2592 with 4, 2 and 1: 541, 517 and 440); and fewer, down to four, while the tiles
 // would leave SMs without work: on a 32^3 grid 16 lines make 64 tiles, four make 256. A tile
 // of long lines (486 points or more) may go on to one line (24 FP64 x lines of 2592 with 4, 2
-// and 1 lines: 185, 114 and 69 µs).
+// and 1 lines: 185, 114 and 69 µs). More than 16 on the shortest lines, whose single butterfly
+// a line (m = 16 and below) would leave half a warp idle, up to 512 points a tile (FP64 y lines
+// of 6 and of 32, 1024 columns, 256 planes, forward, µs: 65 → 43 and 245 → 163). On planes of
+// few columns no tile is twice as wide as the plane, and none of more than 512 points leaves
+// more than a quarter of the columns' number idle (FP64, 6 columns of 1024, 1365 planes, forward
+// and backward: 919 µs with tiles of four, 686 of two; 6 of 24: 40 with eight, 61 with two).
 template <class T, class TI, class TO, bool FWD>
 cudaError_t launch_xform(XformArgs<T> a, cudaStream_t st) {
   if constexpr (sizeof(T) == 4) {
@@ -79,6 +85,11 @@ cudaError_t launch_xform(XformArgs<T> a, cudaStream_t st) {
     return a.axis == 0 ? (a.nlines + L - 1) / L : (long long)a.nz * ((a.nx + L - 1) / L);
   };
   int lg = 4;
+  while (lg < 8 && (a.m << lg) < 512 && tiles(lg + 1) >= 4 * kSMs) ++lg;
+  while (a.axis == 1 && lg > 1 &&
+         ((1 << (lg - 1)) >= a.nx ||
+          ((a.m << lg) > 512 && 4 * (tiles(lg) / a.nz * (1 << lg) - a.nx) > a.nx)))
+    --lg;
   while (lg > 2 && tile_smem(a.m, lg, C) > kBest) --lg;
   while (lg > 0 && tile_smem(a.m, lg, C) > kTwo) --lg;
   while (lg > 0 && tiles(lg) < 2 * kSMs && (lg > 2 || (a.m << lg) >= 486)) --lg;

@@ -1,9 +1,9 @@
 """The line transforms on both sides of the rules that split a pass over the chip.
 
 FP64 x passes of power-of-two lines change their stages at 1216 lines (the passes beyond leave
-the last warp with two of its four lines); lines of other lengths run in tiles of four, two or
-one, by their length and number. Against the oracle, with the tolerances of the solver's other
-parity tests: FP64 1e-12, the refined solve 1e-9 (rtol 1e-10) and FP32 5e-5 of ‖p‖∞.
+the last warp with two of its four lines); lines of other lengths run in tiles of 256 to one, by
+their length and number and the width of a plane. Against the oracle, with the tolerances of the
+solver's other parity tests: FP64 1e-12, the refined solve 1e-9 (rtol 1e-10), FP32 5e-5 of ‖p‖∞.
 """
 
 import numpy as np
@@ -21,6 +21,11 @@ CASES = [(n, 64, 19, b, "P", ("fp64",)) for n, b in ((128, "DD"), (256, "P"), (5
          (1296, 54, 23, "DN", "P", ALL),    # 1242
          (12, 1944, 3, "P", "ND", ALL),     # columns of 972 points, one each
          (108, 2592, 6, "NN", "DD", ALL),   # 648 columns of 1296
+         (2, 1024, 160, "NN", "P", ALL),    # the shortest lines: tiles of 256 rows,
+         (1024, 6, 40, "P", "DD", ALL),     # of 64 columns,
+         (162, 16, 97, "ND", "DN", ALL),    # and a last one of 34
+         (2, 972, 160, "P", "NN", ALL), (6, 1024, 30, "DD", "P", ALL),  # planes narrower than a tile
+         (18, 128, 30, "DN", "ND", ALL),
          (4374, 2, 3, "DD", "NN", ALL), (4608, 6, 60, "P", "NN", ALL), (6, 7776, 2, "DN", "NN", ALL)]
 
 
