@@ -70,8 +70,6 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return r;
 }
 
-// The rectangle's columns run in CTAs of ZB/32 warps spread evenly over the launch (their
-// arithmetic then overlaps the other CTAs' memory traffic instead of filling the SMs first).
 // Loads and stores with an L2 eviction priority (a policy from createpolicy)
 __device__ __forceinline__ float ld_pol(const float* p, uint64_t pol) {
   float v;
@@ -90,6 +88,8 @@ __device__ __forceinline__ void st_pol(float* p, float v, uint64_t pol) {
 template <bool TAB, bool PER, bool ONE>
 __device__ __forceinline__ void zsolve_ckpt(const ZArgs<float>& a, int nlowb) {
   int bulk = blockIdx.x;
+  // The rectangle's columns run in CTAs of ZB/32 warps spread evenly over the launch (their
+  // arithmetic then overlaps the other CTAs' memory traffic instead of filling the SMs first).
   if (nlowb > 0) {
     const int lo = (int)((long long)blockIdx.x * nlowb / gridDim.x);
     const int hi = (int)((long long)(blockIdx.x + 1) * nlowb / gridDim.x);
