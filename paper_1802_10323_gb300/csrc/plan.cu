@@ -320,6 +320,19 @@ struct WsLayout {
   size_t ctrl, partial, info, w, rh, rl, u0, scr_c, scr_u, zlow, total;
 };
 
+// Scratch of the low-wavenumber rectangle of FP32 plans: float pairs (c', d') per row. With a
+// non-periodic z it follows the FP32 columns' checkpoints in the elimination scratch array,
+// which these fill to about an eighth and the rectangle (an eighth of the columns) to half, so
+// that the workspace does not grow with the rectangle; only tiny grids, where the alignment
+// counts, have it behind the other arrays.
+size_t zlow_bytes(const ps_plan* p) { return (size_t)2 * p->nz * p->lowx * p->lowy * sizeof(double); }
+size_t zlow_offset(const ps_plan* p) {  // in the elimination scratch
+  return p->nz <= ZK ? 0 : align256((size_t)zckpt_chunks(p->nz) * p->nx * p->ny * sizeof(float2));
+}
+bool zlow_in_scratch(const ps_plan* p) {
+  return !p->periodic_z && zlow_offset(p) + zlow_bytes(p) <= p->N * sizeof(float);
+}
+
 WsLayout ws_layout(const ps_plan* p) {
   WsLayout L{};
   size_t off = 0;
@@ -345,14 +358,14 @@ WsLayout ws_layout(const ps_plan* p) {
   L.scr_c = off;
   off += align256(p->N * tz);
   L.scr_u = off;
-  const size_t zlow = align256((size_t)2 * p->nz * p->lowx * p->lowy * sizeof(double));
+  const size_t zlow = align256(zlow_bytes(p));
   L.zlow = off;
   if (p->periodic_z) {
     // FP32: the periodic columns' checkpoints fill a small part of this array, and the
     // rectangle's scratch (at most half of it: lowx·lowy ≤ n_x·n_y/8, n_z ≥ 32) follows them
     off += align256(p->N * tz);
     if (zlow) L.zlow = L.scr_u + align256((size_t)zckpt_chunks(p->nz - 1) * p->nx * p->ny * sizeof(float));
-  } else {
+  } else if (!zlow_in_scratch(p)) {
     off += zlow;
   }
   L.total = off;
@@ -412,7 +425,7 @@ ZArgs<T> zargs(const ps_plan* p, T* data, void* ws, const WsLayout& L, const int
     a.ga = (float)p->alpha;
     a.ge0 = (float)p->ge0;
     a.ge1 = (float)p->ge1;
-    a.scr64 = reinterpret_cast<double*>(w + L.zlow);
+    a.scr64 = reinterpret_cast<double*>(zlow_in_scratch(p) ? w + L.scr_c + zlow_offset(p) : w + L.zlow);
   }
   return a;
 }
@@ -431,6 +444,7 @@ ZArgs<T> zargs_t(const ps_plan* p, T* data, void* ws, const WsLayout& L, const i
   if constexpr (sizeof(T) == 4) {
     std::swap(a.lowx, a.lowy);
     std::swap(a.lamx64, a.lamy64);
+    if (zlow_in_scratch(p)) a.scr64 = reinterpret_cast<double*>(reinterpret_cast<char*>(scratch) + zlow_offset(p));
   }
   return a;
 }
