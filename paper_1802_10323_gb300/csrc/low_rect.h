@@ -33,7 +33,8 @@ inline void low_rectangle(const std::vector<double>& lamx, const std::vector<dou
     return tz / (mx[qx] + my[qy] + alpha);
   };
   *lowx = *lowy = 0;
-  if (most < 1 || kappa(0, 0) <= kKappaFew) return;
+  // (couplings beyond FP64's range, whose plan solves nothing, have no rectangle)
+  if (most < 1 || !std::isfinite(tz) || !(kappa(0, 0) > kKappaFew)) return;
   size_t qx = 1, qy = 1;
   for (;;) {
     const double kx = kappa(qx, 0), ky = kappa(0, qy), k = std::max(kx, ky);

@@ -115,3 +115,8 @@ def test_named_grids(rectangles):
         k = _outside(case)[qx, qy]
         print(g, qx, qy, "%.3g" % k)
         assert k <= most, (g, qx, qy, k)
+
+
+def test_no_rectangle_without_finite_couplings(rectangles):
+    lx = T.eigenvalues("NN", 8)
+    assert rectangles([(lx, lx, 0.0, tz) for tz in (np.inf, np.nan, 0.0)]) == [(0, 0)] * 3
